@@ -44,7 +44,8 @@ def listed():
         _case("depth", name="depth-tiny", U=5, V=5, H=64, W=64, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=32,
               fine_labels=81, fine_radius=5),
         # a small camera's light field, host to host: the call of an application that holds no device memory
-        _case("host", name="host-3x3", U=3, V=3, H=376, W=541, dmin=-1.0, dmax=1.0, coarse_labels=32, fine_labels=101),
+        _case("host", name="host-3x3", U=3, V=3, H=376, W=541, dmin=-1.0, dmax=1.0, coarse_labels=32, fine_labels=101,
+              subpixel=2),
         # the 9x9 benchmark light field: its initial pass and its cost volume alone, and the whole method
         # with the soft-argmin read-out
         _case("initial", name="initial-9x9", **bench),
