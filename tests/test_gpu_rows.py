@@ -1,0 +1,65 @@
+"""The row cost kernel (k_fine_rows.cu): its square root against sqrtf, and its blocks, tasks and list
+at sizes where they can go wrong, against the FP64 oracle."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import lfsynth
+import oracle
+from lf_helpers import RTOL, csr_rel_err, gather, pad4_offsets
+
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+def test_sqrt_fast_rounds_as_sqrtf(tmp_path):
+    from paper_1907_13449_gb300 import _build
+    exe = str(tmp_path / "sqrt_check")
+    subprocess.run([_build.nvcc(), "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17", "-I", _build.CSRC,
+                    "-o", exe, os.path.join(HERE, "sqrt_check.cu")], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "0", (r.returncode, r.stdout, r.stderr)
+
+
+# image sizes around the 32 x 8 blocks; windows: nearly equal rows (one task a block), rows that differ
+# by more than a task's span (several tasks, and rows left to the list), and single odd windows
+@pytest.mark.parametrize("channels", [1, 3])
+@pytest.mark.parametrize("H,W", [(1, 1), (7, 33), (8, 32), (9, 31), (17, 65)])
+@pytest.mark.parametrize("kind", ["even", "rows", "mixed"])
+def test_blocks_and_tasks_match_the_oracle(gpu_lib, H, W, kind, channels):
+    import torch
+    G = 121
+    p = lfsynth.LFParams(U=3, V=4, H=H, W=W, census_w=5, dmin=-3.0, dmax=3.0, coarse_labels=16, fine_labels=G,
+                         fine_radius=7, channels=channels)
+    rng = np.random.default_rng(H * 1000 + W + channels)
+    views = lfsynth.random_views(p.U, p.V, H, W, seed=H + W, channels=channels)
+    y, x = np.mgrid[0:H, 0:W]
+    if kind == "even":
+        lo = 40 + (x + y) % 3
+        cnt = np.full((H, W), 31)
+    elif kind == "rows":
+        lo = (y % 8) * 13 + rng.integers(0, 3, (H, W))       # starts 0 .. 93: eight spans in a block
+        cnt = rng.integers(5, 28, (H, W))
+    else:
+        lo = rng.integers(0, G, (H, W))
+        cnt = rng.integers(1, G + 1, (H, W))
+        cnt = np.where(rng.random((H, W)) < 0.7, np.minimum(cnt, 32), cnt)
+    lo = lo.astype(np.int32).reshape(-1)
+    cnt = np.minimum(cnt.reshape(-1), G - lo).astype(np.int32)
+    off = pad4_offsets(cnt)
+    L = gpu_lib.LightFieldDepth(p)
+    L.lo.copy_(torch.from_numpy(lo))
+    L.cnt.copy_(torch.from_numpy(cnt))
+    L.off.copy_(torch.from_numpy(off))
+    L.cost.fill_(float("nan"))
+    L.cost_volume(torch.from_numpy(views).cuda())
+    gpu_lib.lfsgm_sync(L.h)
+    got = L.cost.cpu().numpy()
+    L.close()
+    off_o, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    assert csr_rel_err(gather(got, off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
+    pad = np.ones(off[-1], bool)
+    pad[np.repeat(off[:-1], cnt) + np.arange(cnt.sum()) - np.repeat(np.cumsum(cnt) - cnt, cnt)] = False
+    assert not np.any(got[:off[-1]][pad])                    # padding slots are 0
