@@ -8,9 +8,10 @@
 //  - cost: one warp per run of 32 pixels of a row and one arm, lanes = pixels; the census words
 //    at the labels' nearest shifts come from the edge-padded census (no clamping needed), the
 //    shifts as linear offsets from a per-arm table.
-//  - SGM: one warp per (arm, direction, scanline); the lane's labels stay in registers, the
-//    d-1 / d+1 neighbours across lanes come by one shuffle each way, the predecessor minimum by
-//    one redux.sync; the next 4 cost rows are prefetched; the directions add into the sums
+//  - SGM: one warp per (arm, direction, scanline), above 64 labels, or two scanlines a warp; the
+//    lane's labels stay in registers, the d-1 / d+1 neighbours across lanes come by one shuffle each
+//    way, the predecessor minimum by one redux.sync (two scanlines: two); the next 8 cost rows are
+//    copied ahead into shared memory; the directions add into the sums
 //    with one packed 32/64-bit reduction per lane and step (the host checks that a label's sum
 //    over the paths stays below 2^16, so the 16-bit fields never carry into each other).
 //  - WTA: one warp per 8 (arm, pixel) rows, argmin by one redux.sync over (sum << 8 | label).
@@ -239,7 +240,7 @@ __device__ __forceinline__ void red_words(uint16_t *dst, const uint32_t *v) {
     }
 }
 
-// One warp per (arm, direction, scanline): Eq. 8 in the normalised form
+// A group of 32 / SUB lanes per (arm, direction, scanline): Eq. 8 in the normalised form
 //   L(p,k) = C(p,k) + (min(L'(k), L'(k-1)+P1, L'(k+1)+P1, m+P2) - m),  m = min_k L'(k),
 // L = C where the predecessor is outside the image; sum over directions (Eq. 9).
 // A lane's labels are held as 16-bit pairs in 32-bit words: the minima are per-halfword
@@ -251,6 +252,12 @@ __device__ __forceinline__ void red_words(uint16_t *dst, const uint32_t *v) {
 // below 2^14; labels below 0 read 0x7fff.  The absent labels' sums overflow their halfwords,
 // but a carry only runs into higher, also absent, labels or out of the reduced word, and the
 // WTA reads labels below Lc only.
+// What bounds it: the ALU pipe (byte permutes and halfword minima run at half rate).  The step's
+// minimum is taken with both halves of the word equal (the lane's minimum and its swap), so the
+// warp's 32-bit minimum is the packed pair (m, m) and needs no unpacking; where the labels leave a
+// lane of the group empty (EDGE false), the neighbours of the first and last label come from that
+// lane by a rotation, without selects.  Up to 64 labels a warp runs two scanlines (SUB = 2), so that
+// 32 labels no longer leave half of its lanes idle and 64 labels take four to a lane.
 // Byte costs (C8): a lane's LPT bytes are one 2/4/8-byte load, widened to halfword pairs by one
 // byte permute per pair that also puts kAbsent into the absent labels' halves.
 template <int LPT>
@@ -274,34 +281,43 @@ struct BVec<8> {
     }
 };
 
-template <int LPT, bool C8>
+template <int LPT, bool C8, int SUB, bool EDGE>
 __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict__ cost_v, int H, int W, int Lc,
                                                          int Lcd, const int *__restrict__ pen, int per_arm,
                                                          int narms, uint16_t *__restrict__ sum,
-    const int *__restrict__ order) {
+                                                         const int *__restrict__ order) {
     using CT = typename std::conditional<C8, uint8_t, uint16_t>::type;
     using T = typename std::conditional<C8, typename BVec<LPT>::T, typename CVec<LPT>::T>::type;
     const CT *cost = reinterpret_cast<const CT *>(cost_v);
-    constexpr int NP = LPT / 2;
+    constexpr int NP = LPT / 2, GL = 32 / SUB;               // words of a lane, lanes of a group
+    // Rows in flight, copied asynchronously into a ring per warp (a ring of registers filled by plain
+    // loads waits earlier than its depth says: a warp has six scoreboards for all its loads).
+    constexpr int R = 8;
+    __shared__ __align__(16) T cring[4][R][32];
     constexpr uint32_t SENT = 0x7fff7fffu;
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= per_arm * narms) return;
-    const int arm = gw / per_arm;
-    const int w = gw - arm * per_arm;
-    const int rs = __ldg(order + w);             // longest scanlines first (within the arm)
+    const int lane = threadIdx.x & 31, gl = lane & (GL - 1), wib = threadIdx.x >> 5;
+    const int gw = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * SUB + (SUB == 1 ? 0 : lane / GL);
+    const int total = per_arm * narms;
+    if (gw - (SUB == 1 ? 0 : lane / GL) >= total) return;    // the whole warp
+    const bool have = SUB == 1 || gw < total;                // (the last warp's second group may be empty)
+    const int arm = have ? gw / per_arm : 0;
+    const int rs = __ldg(order + (have ? gw - arm * per_arm : 0));   // longest scanlines first (within the arm)
     const int r = rs & 15, s = rs >> 4;
-    const int dx = dir_dx(r), dy = dir_dy(r);
-    int x, y;
-    scan_start(r, s, H, W, x, y);
-    const int steps = scan_steps(x, y, dx, dy, H, W);
+    int dx, dy, x, y;
+    dir_of(r, dx, dy);
+    scan_start_d(dx, dy, s, H, W, x, y);
+    const int steps = have ? scan_steps(x, y, dx, dy, H, W) : 0;
+    int most = steps, least = steps;                         // of the warp's groups
+    if (SUB == 2) {
+        const int other = __shfl_xor_sync(0xffffffffu, steps, 16);
+        most = max(most, other);
+        least = min(least, other);
+    }
     const size_t N = (size_t)H * W;
-    const int k0 = lane * LPT;
+    const int k0 = gl * LPT;
     const bool act = k0 < Lcd;
-    const CT *C = cost + (size_t)arm * N * Lcd + k0;
-    uint16_t *S = sum + (size_t)arm * N * Lcd + k0;
     const uint32_t P1 = (uint32_t)__ldg(pen + 2 * arm), P2 = (uint32_t)__ldg(pen + 2 * arm + 1);
-    const uint32_t P1P1 = P1 * 0x10001u;
+    const uint32_t P1P1 = P1 * 0x10001u, PQ = (P2 - P1) * 0x10001u;
     constexpr uint32_t ABS2 = (uint32_t)kAbsent * 0x10001u;
     // byte costs: one byte permute per label pair widens two bytes to halfwords and puts kAbsent
     // (= 0x2000: bytes 0x00, 0x20 of the constant operand, selectors 4 and 5) into the halves of
@@ -314,18 +330,25 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
         const uint32_t hi = (k0 + 2 * j + 1 < Lc && act) ? (uint32_t)(b + 1) | (4u << 4) : 0x54u;
         bsel[j] = lo | (hi << 8);
     }
-    // cost and sum pointers step along the scanline; the cost rows of the next four steps are in
-    // flight (a ring of four registers, indexed statically by unrolling the steps by four)
+    // cost and sum pointers step along the scanline; row t goes to ring slot t mod R
     const long long dstep = ((long long)dy * W + dx) * Lcd;
-    const CT *pc = C + ((long long)y * W + x) * Lcd;
-    uint16_t *ps = S + ((long long)y * W + x) * Lcd;
-    auto ld = [&](int t) {
-        T v;
-        if constexpr (C8) v = T{};
-        else v = CVec<LPT>::fill(ABS2);
-        if (act && t < steps) v = __ldg(reinterpret_cast<const T *>(pc + (long long)t * dstep));
-        return v;
+    const size_t first = ((size_t)arm * N + (size_t)y * W + x) * Lcd + k0;
+    const CT *pc = cost + first;                                     // the next row to load
+    uint16_t *ps = sum + first;
+    const unsigned cdst = (unsigned)__cvta_generic_to_shared(&cring[wib][0][lane]);
+    // (two-byte rows, LPT = 2: even lanes copy for their neighbour too)
+    const bool loads = sizeof(T) == 2 ? act && (gl & 1) == 0 : act;
+    auto ld = [&](int i, bool in) {                                  // in: the scanline has this row
+        if (loads && in)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(cdst + i * 32 * (unsigned)sizeof(T)), "l"(pc),
+                         "n"(sizeof(T) < 4 ? 4 : sizeof(T)) : "memory");
+        pc += dstep;
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    if constexpr (!C8) {
+        if (!act)
+            for (int i = 0; i < R; i++) cring[wib][i][lane] = CVec<LPT>::fill(ABS2);
+    }
     auto words = [&](const T &v, uint32_t *c) {
         if constexpr (C8) {
             uint32_t src[(NP + 1) / 2];
@@ -336,54 +359,64 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
             words_of<LPT>(v, c);
         }
     };
-    T ring[4] = {ld(0), ld(1), ld(2), ld(3)};
+    for (int i = 0; i < R; i++) ld(i, i < steps);
     uint32_t L[NP];
-    uint32_t m;
-    auto finish = [&](const uint32_t *Ln) {       // warp minimum, packed reduction, carry the row
+    uint32_t mm = 0;                                                 // (m, m)
+    auto finish = [&](const uint32_t *Ln, bool on) {   // group minimum, packed reduction, carry the row
         uint32_t q = Ln[0];
 #pragma unroll
-        for (int j = 1; j < NP; j++) q = __vimin3_u16x2(q, Ln[j], Ln[j]);
-        m = __reduce_min_sync(0xffffffffu, min(q & 0xffffu, q >> 16));
-        if (act) red_words<LPT>(ps, Ln);
+        for (int j = 1; j < NP; j++) q = __vminu2(q, Ln[j]);
+        q = __vminu2(q, __byte_perm(q, 0, 0x1032));                  // both halves: the lane's minimum
+        if constexpr (SUB == 1) {
+            mm = __reduce_min_sync(0xffffffffu, q);
+        } else {
+            const uint32_t m0 = __reduce_min_sync(0xffffffffu, lane < 16 ? q : 0xffffffffu);
+            const uint32_t m1 = __reduce_min_sync(0xffffffffu, lane < 16 ? 0xffffffffu : q);
+            mm = lane < 16 ? m0 : m1;
+        }
+        if (act && on) red_words<LPT>(ps, Ln);
         ps += dstep;
 #pragma unroll
         for (int j = 0; j < NP; j++) L[j] = Ln[j];
     };
-    {   // path start: L = C
-        uint32_t Ln[NP];
-        words(ring[0], Ln);
-        ring[0] = ld(4);
-        finish(Ln);
-    }
-    for (int t0 = 1; t0 < steps; t0 += 4) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const int t = t0 + k;
-            if (t >= steps) break;
-            const int slot = (1 + k) & 3;          // step t's row sits in ring[t % 4]
-            uint32_t c[NP];
-            words(ring[slot], c);
-            ring[slot] = ld(t + 4);
-            uint32_t left = __shfl_up_sync(0xffffffffu, L[NP - 1], 1);
-            uint32_t right = __shfl_down_sync(0xffffffffu, L[0], 1);
-            if (lane == 0) left = SENT;
-            if (lane == 31) right = SENT;
-            // min(L'(k), L'(k-1)+P1, L'(k+1)+P1, m+P2) = min(L'(k), min(L'(k-1), L'(k+1), m+P2-P1) + P1):
-            // one 3-way and one add-then-min per halfword pair (DPX)
-            const uint32_t mm = __byte_perm(m, 0, 0x1010), mq = __byte_perm(m + P2 - P1, 0, 0x1010);
-            uint32_t Ln[NP];
-#pragma unroll
-            for (int j = 0; j < NP; j++) {
-                const uint32_t pw = (j == 0) ? left : L[j - 1];
-                const uint32_t nw = (j == NP - 1) ? right : L[j + 1];
-                const uint32_t lm = __byte_perm(pw, L[j], 0x5432);    // labels 2j-1, 2j
-                const uint32_t rp = __byte_perm(L[j], nw, 0x5432);    // labels 2j+1, 2j+2
-                const uint32_t u = __viaddmin_u16x2(__vimin3_u16x2(lm, rp, mq), P1P1, L[j]);
-                Ln[j] = c[j] + (u - mm);
-            }
-            finish(Ln);
+    // one step on the row in ring slot i (the oldest copy), whose slot then takes the row R steps on
+    auto step = [&](int i, bool start, bool in, bool on) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(R - 1) : "memory");
+        if constexpr (sizeof(T) == 2) __syncwarp();
+        uint32_t c[NP];
+        words(cring[wib][i][lane], c);
+        ld(i, in);
+        if (start) {   // path start: L = C
+            finish(c, on);
+            return;
         }
+        uint32_t left = __shfl_sync(0xffffffffu, L[NP - 1], gl + GL - 1, GL);
+        uint32_t right = __shfl_sync(0xffffffffu, L[0], gl + 1, GL);
+        if (EDGE && gl == 0) left = SENT;
+        if (EDGE && gl == GL - 1) right = SENT;
+        // min(L'(k), L'(k-1)+P1, L'(k+1)+P1, m+P2) = min(L'(k), min(L'(k-1), L'(k+1), m+P2-P1) + P1):
+        // one 3-way and one add-then-min per halfword pair (DPX)
+        const uint32_t mq = mm + PQ;
+        uint32_t Ln[NP];
+#pragma unroll
+        for (int j = 0; j < NP; j++) {
+            const uint32_t pw = (j == 0) ? left : L[j - 1];
+            const uint32_t nw = (j == NP - 1) ? right : L[j + 1];
+            const uint32_t lm = __byte_perm(pw, L[j], 0x5432);    // labels 2j-1, 2j
+            const uint32_t rp = __byte_perm(L[j], nw, 0x5432);    // labels 2j+1, 2j+2
+            const uint32_t u = __viaddmin_u16x2(__vimin3_u16x2(lm, rp, mq), P1P1, L[j]);
+            Ln[j] = c[j] + u - mm;
+        }
+        finish(Ln, on);
+    };
+    step(0, true, R < steps, have);
+    // R steps at a time, as long as both groups have all of them and the rows to load; then the rest
+    int t0 = 1;
+    for (; t0 + 2 * R <= least; t0 += R) {
+#pragma unroll
+        for (int k = 0; k < R; k++) step((1 + k) & (R - 1), false, true, true);   // (t0 = 1 mod R)
     }
+    for (int t = t0; t < most; t++) step(t & (R - 1), false, t + R < steps, SUB == 1 || t < steps);
 }
 
 // WTA over the path sums (Eq. 10): lowest label on ties (the key is sum << 8 | label).
@@ -469,15 +502,24 @@ cudaError_t launch_coarse_sgm(cudaStream_t s, const void *cost, bool cost8, int 
                               const int *pen, uint16_t *sum, const int *order, int paths) {
     const ScanTable st = make_scan_table(H, W, paths);
     const int Lcd = coarse_stride(Lc);
-    const long long warps = (long long)st.cum[paths] * narms;
+    // labels per lane and scanlines per warp: with 32 labels, one scanline of two labels a lane in a warp
+    // took 317 us on 3x3 x 376x541, two scanlines 150 us
+    const int lpt = Lc <= 32 ? 2 : Lc <= 128 ? 4 : 8, sub = Lc <= 64 ? 2 : 1;
+    const bool edge = Lcd == lpt * 32 / sub;                          // no lane of a group is empty
+    const long long warps = ((long long)st.cum[paths] * narms + sub - 1) / sub;
     const int block = 128;
     const unsigned grid = (unsigned)((warps * 32 + block - 1) / block);
-#define LFSGM_SGM(LPT, B) coarse_sgm_kernel<LPT, B><<<grid, block, 0, s>>>(cost, H, W, Lc, Lcd, pen, st.cum[paths], narms, sum, order)
-    switch (coarse_lpt(Lc)) {
-    case 2: if (cost8) LFSGM_SGM(2, true); else LFSGM_SGM(2, false); break;
-    case 4: if (cost8) LFSGM_SGM(4, true); else LFSGM_SGM(4, false); break;
-    default: if (cost8) LFSGM_SGM(8, true); else LFSGM_SGM(8, false); break;
-    }
+#define LFSGM_SGM(LPT, B, SUB, E) coarse_sgm_kernel<LPT, B, SUB, E><<<grid, block, 0, s>>>(cost, H, W, Lc, Lcd, pen, st.cum[paths], narms, sum, order)
+#define LFSGM_SGM4(LPT, SUB)                                                                    \
+    do {                                                                                        \
+        if (cost8) { if (edge) LFSGM_SGM(LPT, true, SUB, true); else LFSGM_SGM(LPT, true, SUB, false); } \
+        else { if (edge) LFSGM_SGM(LPT, false, SUB, true); else LFSGM_SGM(LPT, false, SUB, false); }     \
+    } while (0)
+    if (lpt == 2) LFSGM_SGM4(2, 2);
+    else if (sub == 2) LFSGM_SGM4(4, 2);
+    else if (lpt == 4) LFSGM_SGM4(4, 1);
+    else LFSGM_SGM4(8, 1);
+#undef LFSGM_SGM4
 #undef LFSGM_SGM
     return cudaGetLastError();
 }
