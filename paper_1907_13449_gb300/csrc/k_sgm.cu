@@ -13,7 +13,10 @@
 // The step is the normalised recurrence
 //   L(p,g) = C(p,g) + (min(L'(g), L'(g-1)+P1, L'(g+1)+P1, m+P2) - m),   m = min L',
 // and the predecessor minimum m is one redux.sync.min.f32 per pixel.  The 8 or 16 directions run
-// concurrently and add into agg (zeroed by the caller) with float atomics.  Optionally the few
+// concurrently and add into agg (zeroed by the caller) with float atomics.  A run of equal windows of
+// 33 to 128 labels (whole-range searches) keeps the predecessor's row in registers, four consecutive
+// labels a lane: one vector load and one vector reduction a step, the neighbours across lanes by two
+// shuffles (7x1 x 555x650, 121 labels: 295 instructions a step in shared-memory chunks, 956 us).  Optionally the few
 // scanlines that cross many wide windows (a speed knob) run on all the warps of a CTA each, which
 // share the wide steps' chunks (sgm_scanline SPLIT); a small kernel lists them first.
 //
@@ -118,7 +121,81 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
     bool in_smem = false;                      // the predecessor row is in bufA (after a general step)
     int gpar = 0;                              // SPLIT: which half of xm this general step uses
     int k = 0;
+    // the block of metadata after the one that ends at step k (a multiple of 32)
+    auto next_block = [&]() {
+        cw = nw;
+        co = no;
+        if (k + 32 < len) {
+            fetch(k + 32, nw, no);
+        } else {
+            nw = 0;
+            no = 0;
+        }
+        meta[(k + 32 + lane) & 63] = make_int2(nw, no);   // the slots of the block just finished
+        __syncwarp();
+    };
     while (k < len) {
+        if constexpr (!REC && !SPLIT) {
+            // a run of windows equal to the predecessor's, 33 to 128 labels, after a general step
+            if (in_smem && pn > 32 && pn <= 128 && meta[k & 63].x == (plo | (pn << 16))) {
+                const int pw = meta[k & 63].x, j0 = 4 * lane;
+                // the labels j0 .. j0 + 3 that the window has (the padding slots of a row are never used)
+                const bool h0 = j0 < pn, h1 = j0 + 1 < pn, h2 = j0 + 2 < pn, h3 = j0 + 3 < pn;
+                float v0 = h0 ? bufA[j0] : INF, v1 = h1 ? bufA[j0 + 1] : INF;
+                float v2 = h2 ? bufA[j0 + 2] : INF, v3 = h3 ? bufA[j0 + 3] : INF;
+                const float4 *cb = reinterpret_cast<const float4 *>(cost) + lane;
+                float *ab = agg + j0;
+                const float4 none = make_float4(INF, INF, INF, INF);
+                // cost rows two steps ahead; a step that is not in the run loads nothing
+                auto row = [&](int2 mt) { return h0 && mt.x == pw ? __ldg(cb + mt.y) : none; };
+                int2 mt = meta[k & 63], mt1 = meta[(k + 1) & 63];
+                float4 c = row(mt), c1 = row(mt1);
+                for (;;) {
+                    const int2 mt2 = meta[(k + 2) & 63];
+                    const float4 c2 = row(mt2);
+                    if (!h1) c.y = INF;
+                    if (!h2) c.z = INF;
+                    if (!h3) c.w = INF;
+                    const float vl = __shfl_up_sync(0xffffffffu, v3, 1), vr = __shfl_down_sync(0xffffffffu, v0, 1);
+                    const float left = lane == 0 ? INF : vl, right = lane == 31 ? INF : vr;
+                    const float q = m + P2;
+                    // absent labels: c = +inf, so L = +inf
+                    const float n0 = c.x + (fminf(fminf(q, v0), fminf(left, v1) + P1) - m);
+                    const float n1 = c.y + (fminf(fminf(q, v1), fminf(v0, v2) + P1) - m);
+                    const float n2 = c.z + (fminf(fminf(q, v2), fminf(v1, v3) + P1) - m);
+                    const float n3 = c.w + (fminf(fminf(q, v3), fminf(v2, right) + P1) - m);
+                    if (h0) {
+                        const float a0 = det_addend(n0, c.x + P2, mk);
+                        const float a1 = h1 ? det_addend(n1, c.y + P2, mk) : 0.f;
+                        const float a2 = h2 ? det_addend(n2, c.z + P2, mk) : 0.f;
+                        const float a3 = h3 ? det_addend(n3, c.w + P2, mk) : 0.f;
+                        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
+                                     ::"l"(ab + 4ll * mt.y), "f"(a0), "f"(a1), "f"(a2), "f"(a3) : "memory");
+                    }
+                    v0 = n0;
+                    v1 = n1;
+                    v2 = n2;
+                    v3 = n3;
+                    m = warp_min(fminf(fminf(n0, n1), fminf(n2, n3)));
+                    k++;
+                    if ((k & 31) == 0 && k < len) next_block();
+                    if (mt1.x != pw || k >= len) break;
+                    mt = mt1;
+                    c = c1;
+                    c1 = c2;
+                    mt1 = mt2;
+                }
+                // the row back to shared memory for what follows
+                __syncwarp();
+                if (h0) bufA[j0] = v0;
+                if (h1) bufA[j0 + 1] = v1;
+                if (h2) bufA[j0 + 2] = v2;
+                if (h3) bufA[j0 + 3] = v3;
+                __syncwarp();
+                prev = lane < pn ? bufA[lane] : INF;
+                continue;
+            }
+        }
         const int kb = k & ~31;
         const int kbend = min(kb + 32, len);
         // steps of this block that need the general form: invalid or wider than 32 labels
@@ -318,18 +395,7 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
             }
             k++;
         }
-        if ((k & 31) == 0 && k < len) {       // next block of metadata
-            cw = nw;
-            co = no;
-            if (k + 32 < len) {
-                fetch(k + 32, nw, no);
-            } else {
-                nw = 0;
-                no = 0;
-            }
-            meta[(k + 32 + lane) & 63] = make_int2(nw, no);   // the slots of the block just finished
-            __syncwarp();
-        }
+        if ((k & 31) == 0 && k < len) next_block();
     }
 }
 
