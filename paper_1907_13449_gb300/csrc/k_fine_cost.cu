@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(32 * kListWarps, C == 3 ? 12 : (LEAN ? 16 : 12
                                                       const int *__restrict__ cnt,
                                                       const long long *__restrict__ off, float wl2, float wc,
                                                       float *__restrict__ cost, const int2 *__restrict__ list,
-                                                      const int *__restrict__ count) {
+                                                      const int *__restrict__ count,
+                                                      const int *__restrict__ large) {
+    if (large && __ldg(large) == 0) return;              // census_list has done the list
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     const size_t HWp = (size_t)Hp * Wp;
@@ -157,6 +159,143 @@ __global__ void __launch_bounds__(32 * kListWarps, C == 3 ? 12 : (LEAN ? 16 : 12
 }
 
 
+// The cost without the l2 term (w_l2 = 0, the paper's census-only cost of real scenes; grey), while the
+// views are small enough that 0 x l2 is 0 (`large` is not set: with a NaN or an infinity among the
+// samples 0 x l2 is NaN, so the full list runs then).  7x1 x 555x650, 121 labels, every window the whole
+// range: 722 us in the full list; 495 us in census_list alone (a few views an item: its loads' latency);
+// most of it in census_runs.
+//
+// Runs of 32 pixels of a row whose windows are all the whole range (marked by row_tasks_kernel): one
+// warp per run, lane = pixel.  A label's shift is the same for every pixel and changes only every few
+// labels, so a view's Hamming distance is a step function of the label (as in the coarse cost): a word
+// read, coalesced over the pixels, and a popcount only at the steps, added to a difference column in
+// shared memory (two labels a word), prefix-summed, and the rows written through a 32 x 32 tile.
+constexpr int kRunLabels = 96, kRunWarps = 4;
+__global__ void __launch_bounds__(32 * kRunWarps) census_runs(const uint64_t *__restrict__ cen_pad, int P, int Wp,
+                                                              int Hp, const int *__restrict__ ctab, int G, int nviews,
+                                                              int H, int W, int ref,
+                                                              const unsigned char *__restrict__ marks,
+                                                              const long long *__restrict__ off, float wc,
+                                                              float *__restrict__ cost) {
+    __shared__ int cdiff[kRunWarps][kRunLabels / 2][32];
+    __shared__ float tile[kRunWarps][32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int bx = (W + 31) >> 5;
+    const int run = blockIdx.x * kRunWarps + w;              // row-major over (row, run of the row)
+    if (run >= bx * H || !__ldg(marks + run)) return;
+    const int y = run / bx, x0 = (run - y * bx) << 5, x = min(x0 + lane, W - 1);
+    const size_t HWp = (size_t)Hp * Wp, base = (size_t)(y + P) * Wp + (x + P);
+    const int npx = min(32, W - x0);
+    const long long o = __ldg(off + (size_t)y * W + x);
+    const int npad = (int)min((long long)((G + 3) & ~3), __ldg(off + (size_t)y * W + x + 1) - o);
+    const uint64_t cr = __ldg(cen_pad + (size_t)ref * HWp + base);
+    int *cd = &cdiff[w][0][lane];
+    for (int g0 = 0; g0 < G; g0 += kRunLabels) {
+        const int ng = min(kRunLabels, G - g0);
+#pragma unroll 4
+        for (int i = 0; i < kRunLabels / 2; i++) cd[32 * i] = 0;
+        for (int v = 0; v < nviews; v++) {
+            if (v == ref) continue;
+            const uint64_t *q = cen_pad + (size_t)v * HWp + base;
+            const int *ot = ctab + (size_t)v * G + g0;
+            int hp = 0, oprev = 0;
+            for (int k0 = 0; k0 < ng; k0 += 32) {
+                const int k = k0 + lane;
+                const int ov = k < ng ? __ldg(ot + k) : 0;
+                const int up = __shfl_up_sync(0xffffffffu, ov, 1);
+                const int before = lane == 0 ? oprev : up;
+                unsigned steps = __ballot_sync(0xffffffffu, k < ng && (k == 0 || ov != before));
+                oprev = __shfl_sync(0xffffffffu, ov, 31);
+                // the steps four at a time: their word loads are issued together
+                while (steps) {
+                    int bs[4];
+                    uint64_t wv[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        bs[u] = steps ? __ffs(steps) - 1 : -1;          // warp-uniform
+                        steps &= steps - 1;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int so = __shfl_sync(0xffffffffu, ov, bs[u] & 31);
+                        wv[u] = bs[u] >= 0 ? __ldg(q + so) : 0ull;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        if (bs[u] < 0) break;
+                        const int h = __popcll(cr ^ wv[u]);
+                        const int kb = k0 + bs[u];
+                        cd[32 * (kb >> 1)] += (int)((unsigned)(h - hp) << (16 * (kb & 1)));
+                        hp = h;
+                    }
+                }
+            }
+        }
+        int sum = 0;
+        for (int k0 = 0; k0 < ng; k0 += 32) {
+#pragma unroll 4
+            for (int k = 0; k < 32; k += 2) {
+                // the word holds d(k) + d(k+1) 2^16 (two's complement, |d| < 2^15): split it exactly
+                const int wd = cd[32 * ((k0 + k) >> 1)];
+                const int d0 = (int)(short)(wd & 0xffff);
+                sum += d0;
+                tile[w][lane][k] = wc * (float)sum;
+                sum += (wd - d0) >> 16;
+                tile[w][lane][k + 1] = wc * (float)sum;
+            }
+            __syncwarp();
+            const int j = g0 + k0 + lane;
+#pragma unroll 4
+            for (int q = 0; q < npx; q++) {
+                const long long oq = __shfl_sync(0xffffffffu, o, q);
+                const int nq = __shfl_sync(0xffffffffu, npad, q);
+                if (j < nq) cost[oq + j] = j < G ? tile[w][q][lane] : 0.f;
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// The other items: one warp per (pixel, 32-label chunk); per view a lane reads its label's offset
+// (ctab: ny Wp + nx) and one census word.
+__global__ void __launch_bounds__(32 * kListWarps) census_list(const uint64_t *__restrict__ cen_pad, int P, int Wp,
+                                                               int Hp, const int *__restrict__ ctab, int G, int nviews,
+                                                               int W, int ref, const int *__restrict__ lo,
+                                                               const int *__restrict__ cnt,
+                                                               const long long *__restrict__ off, float wc,
+                                                               float *__restrict__ cost, const int2 *__restrict__ list,
+                                                               const int *__restrict__ count,
+                                                               const int *__restrict__ large) {
+    if (__ldg(large)) return;
+    const int lane = threadIdx.x & 31;
+    const int warps = (gridDim.x * blockDim.x) >> 5;
+    const size_t HWp = (size_t)Hp * Wp;
+    const int total = *count;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += warps) {
+        const int2 item = __ldg(list + t);
+        const int p = item.x, chunk = item.y;
+        const int l0 = __ldg(lo + p), n = __ldg(cnt + p);
+        const long long o = __ldg(off + p), row = __ldg(off + p + 1) - o;
+        if (!window_ok(l0, n, G, row, nullptr)) continue;      // items are pushed for valid windows only
+        const int npad = (int)min((long long)((n + 3) & ~3), row);
+        const int j = chunk * 32 + lane;
+        const int x = p % W, y = p / W;
+        const size_t base = (size_t)(y + P) * Wp + (x + P);
+        int sc = 0;
+        if (j < n) {
+            const uint64_t cr = __ldg(cen_pad + (size_t)ref * HWp + base);
+            const int *tg = ctab + l0 + j;
+            const uint64_t *q = cen_pad + base;
+            auto view = [&](int v) { return __popcll(cr ^ __ldg(q + (size_t)v * HWp + __ldg(tg + (size_t)v * G))); };
+            int v = 0;
+            // (the reference view's own distance, at shift 0, is 0)
+            for (; v + 4 <= nviews; v += 4) sc += view(v) + view(v + 1) + view(v + 2) + view(v + 3);
+            for (; v < nviews; v++) sc += view(v);
+        }
+        if (j < npad) cost[o + j] = j < n ? wc * (float)sc : 0.f;
+    }
+}
+
 __global__ void list_all_kernel(const int *__restrict__ lo, const int *__restrict__ cnt,
                                 const long long *__restrict__ off, int G, int2 *list, int *count, int N,
                                 int *status, int min_cnt) {
@@ -176,7 +315,8 @@ cudaError_t launch_list_all(cudaStream_t s, const int *lo, const int *cnt, const
 cudaError_t launch_fine_cost_list(cudaStream_t s, const float *views_pad, const uint64_t *cen_pad, int P, int Wp,
                                   int Hp, const int4 *ltab, int G, int nviews, int C, int W, int ref,
                                   const int *lo, const int *cnt, const long long *off, float wl2, float wc,
-                                  float *cost, const int2 *list, const int *count, int ctas_per_sm) {
+                                  float *cost, const int2 *list, const int *count, int ctas_per_sm,
+                                  const int *large) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -194,7 +334,29 @@ cudaError_t launch_fine_cost_list(cudaStream_t s, const float *views_pad, const 
         k = max(k, 1);
     }
     kern<<<sms * k, 32 * kListWarps, 0, s>>>(views_pad, cen_pad, P, Wp, Hp, ltab, G, nviews, W, ref, lo, cnt, off, wl2,
-                                             wc, cost, list, count);
+                                             wc, cost, list, count, large);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_census_runs(cudaStream_t s, const uint64_t *cen_pad, int P, int Wp, int Hp, const int *ctab, int G,
+                               int nviews, int H, int W, int ref, const unsigned char *marks, const long long *off,
+                               float wc, float *cost) {
+    const long long runs = (long long)((W + 31) / 32) * H;
+    census_runs<<<(unsigned)((runs + kRunWarps - 1) / kRunWarps), 32 * kRunWarps, 0, s>>>(
+        cen_pad, P, Wp, Hp, ctab, G, nviews, H, W, ref, marks, off, wc, cost);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_census_list(cudaStream_t s, const uint64_t *cen_pad, int P, int Wp, int Hp, const int *ctab, int G,
+                               int nviews, int W, int ref, const int *lo, const int *cnt, const long long *off, float wc,
+                               float *cost, const int2 *list, const int *count, const int *large) {
+    int dev = 0, sms = 0, k = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, census_list, 32 * kListWarps, 0);
+    if (e != cudaSuccess) return e;
+    census_list<<<sms * max(k, 1), 32 * kListWarps, 0, s>>>(cen_pad, P, Wp, Hp, ctab, G, nviews, W, ref, lo, cnt, off, wc,
+                                                            cost, list, count, large);
     return cudaGetLastError();
 }
 

@@ -109,7 +109,9 @@ __global__ void __launch_bounds__(32 * kBlkH) row_tasks_kernel(const int *__rest
                                                                const long long *__restrict__ off, int G, int H, int W,
                                                                int kw, int kwt, int nblk, RowTask *__restrict__ tasks,
                                                                int *__restrict__ extra, int2 *__restrict__ list,
-                                                               int *__restrict__ list_count, int *__restrict__ status) {
+                                                               int *__restrict__ list_count, int *__restrict__ status,
+                                                               const int *__restrict__ large,
+                                                               unsigned char *__restrict__ marks) {
     __shared__ int sg0[kBlkH], shi[kBlkH];
     __shared__ unsigned sm[kBlkH];
     const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
@@ -125,6 +127,13 @@ __global__ void __launch_bounds__(32 * kBlkH) row_tasks_kernel(const int *__rest
             nar = n <= 32;
             todo = !nar;
         }
+    }
+    if (marks && y < H) {                                 // warp-uniform
+        // a run of whole-range windows (wider than 32 labels) for census_runs
+        const bool whole = x >= W || (todo && l == 0 && n == G);
+        const bool all = __ballot_sync(0xffffffffu, whole) == 0xffffffffu && !__ldg(large);
+        if (lane == 0) marks[(size_t)y * bx + b % bx] = all;
+        if (all) todo = false;
     }
     unsigned left = __ballot_sync(0xffffffffu, nar);
     int best = 0, g0 = 0;
@@ -673,12 +682,12 @@ bool encode_fine_rows_maps(RowPlanHost *ph, const float *views_pad, const uint64
 
 cudaError_t launch_row_tasks(cudaStream_t s, const RowPlanHost *ph, int G, int H, int W, const int *lo, const int *cnt,
                              const long long *off, RowTask *tasks, int *extra, int *status, int2 *list,
-                             int *list_count) {
+                             int *list_count, const int *large, unsigned char *marks) {
     RowPlan pl;
     memcpy(&pl, ph->raw, sizeof(pl));
     const int nblk = row_blocks(H, W);
     row_tasks_kernel<<<nblk, 32 * kBlkH, 0, s>>>(lo, cnt, off, G, H, W, pl.kw, pl.kwt, nblk, tasks, extra, list, list_count,
-                                                    status);
+                                                    status, large, marks);
     return cudaGetLastError();
 }
 

@@ -70,6 +70,7 @@ struct lfsgm_ctx {
     int4 *d_rowheads = nullptr;           // and their tile headers
     int *d_order = nullptr;               // SGM scanlines, longest first
     int4 *d_ltab = nullptr;               // taps as linear offsets in the padded images (list kernel)
+    int *d_ctab = nullptr;                // the census offsets alone (grey without the l2 term)
     int *d_otab = nullptr;       // coarse census offsets per (arm view, label), see CoarseArms
     CoarseArms ca{};
     int *d_armviews = nullptr;   // [4][kMaxArmViews]
@@ -87,8 +88,9 @@ struct lfsgm_ctx {
     uint16_t *csum = nullptr;
     int *maps = nullptr, *F0 = nullptr, *F1 = nullptr, *cntpad = nullptr;
     int2 *wide_list = nullptr;         // (pixel, 32-label chunk) items for the list kernel
-    int *wide_count = nullptr;         // list items, then the row kernel's further tasks
+    int *wide_count = nullptr;         // list items, the row kernel's further tasks; [2]: a large value in the views
     RowTask *row_tasks = nullptr;      // label ranges of the row kernel's blocks
+    unsigned char *marks = nullptr;    // runs of whole-range windows (census_only)
     RowPlanHost rows{};                // row-sweep cost kernel plan + tensor maps
     bool rows_maps = false;            // tensor maps encoded for the bound workspace
     float *views_pad = nullptr;        // edge-replicated padded copies (workspace)
@@ -247,6 +249,11 @@ lfsgm_status ensure_workspace(lfsgm_ctx *h) {
     return bind_workspace(h, p, bytes, true);
 }
 
+// The cost is the census term alone, grey: the list skips the l2 samples unless a view holds a value
+// whose samples could make 0 x l2 a NaN (flagged with the census).
+bool census_only(const lfsgm_ctx *h) { return h->cfg.w_l2 == 0.f && h->C == 1; }
+int *large_flag(lfsgm_ctx *h) { return census_only(h) ? h->wide_count + 2 : nullptr; }
+
 int max_arm_views(const lfsgm_ctx *h) {
     int m = 0;
     for (int a = 0; a < h->arms.n_arms; a++) m = std::max(m, h->arms.nv[a]);
@@ -285,8 +292,9 @@ lfsgm_status bind_workspace(lfsgm_ctx *h, void *dptr, size_t bytes, bool owned) 
     h->F1 = (int *)take(N * 4);
     h->cntpad = (int *)take(N * 4);
     h->wide_list = (int2 *)take(N * (size_t)((h->cfg.fine_labels + 31) / 32) * 8);
-    h->wide_count = (int *)take(8);
+    h->wide_count = (int *)take(12);
     h->row_tasks = (RowTask *)take(8 * (size_t)row_blocks(h->cfg.H, h->cfg.W) * sizeof(RowTask));
+    h->marks = (unsigned char *)take((size_t)((h->cfg.W + 31) / 32) * h->cfg.H);
     h->armsum = (unsigned long long *)take(4 * 8);
     h->cpen = (int *)take(8 * 4);
     h->fpen = (float *)take(2 * 4);
@@ -434,6 +442,11 @@ lfsgm_status lfsgm_create(const lfsgm_config *cfg, void *stream, lfsgm_handle *o
             ltab[i] = e;
         }
         ALLOC_COPY(h->d_ltab, ltab);
+        if (census_only(h)) {
+            std::vector<int> ctab(ltab.size());
+            for (size_t i = 0; i < ltab.size(); i++) ctab[i] = ltab[i].y;
+            ALLOC_COPY(h->d_ctab, ctab);
+        }
     }
     if (h->rows.ok) {
         std::vector<unsigned char> desc;
@@ -466,6 +479,7 @@ lfsgm_status lfsgm_destroy(lfsgm_handle h) {
     cudaFree(h->d_rowheads);
     cudaFree(h->d_order);
     cudaFree(h->d_ltab);
+    cudaFree(h->d_ctab);
     cudaFree(h->d_otab);
     cudaFree(h->d_armviews);
     cudaFree(h->d_sel_cross);
@@ -495,8 +509,9 @@ lfsgm_status lfsgm_workspace_size(lfsgm_handle h, size_t *bytes) {
     b += align256(4 * N * 4);                       // maps
     b += 3 * align256(N * 4);                       // F0, F1, padded counts
     b += align256(N * (size_t)((h->cfg.fine_labels + 31) / 32) * 8);   // (pixel, chunk) list
-    b += align256(8);                               // list and task counts
+    b += align256(12);                              // list and task counts, large-value flag
     b += align256(8 * (size_t)row_blocks(h->cfg.H, h->cfg.W) * sizeof(RowTask));
+    b += align256((size_t)((h->cfg.W + 31) / 32) * h->cfg.H);   // run marks
     b += align256(4 * 8) + align256(8 * 4) + align256(2 * 4);
     b += align256(2 * kPartialBlocks * 8) + 2 * align256(4);   // partials; status word and ticket
     b += align256((size_t)scan_tiles(h->N) * 8);    // offset-scan tile sums
@@ -603,9 +618,11 @@ lfsgm_status lfsgm_initial_disparity(lfsgm_handle h, const float *views, int32_t
     int *fin = h->F0, *fout = h->F1;
     cudaError_t e = cudaSuccess;
     if (!c.boundless) {   // boundary-less: no initial map, the windows kernel writes whole-range windows
+        if (census_only(h)) e = cudaMemsetAsync(large_flag(h), 0, 4, s);
+        if (e != cudaSuccess) return cuda_fail(h, e, "memset");
         LFSGM_TRY(run(h, "census_cross", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
-                                     h->d_sel_cross, h->n_sel_cross, h->cen_pad, h->views_pad);
+                                     h->d_sel_cross, h->n_sel_cross, h->cen_pad, h->views_pad, large_flag(h));
         }));
         e = cudaMemsetAsync(h->armsum, 0, 4 * 8, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->csum, 0, (size_t)A * N * h->Lcd * 2, s);
@@ -662,14 +679,18 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
     const lfsgm_config &c = h->cfg;
     cudaStream_t s = h->stream;
     if (!cross_done) {
+        if (census_only(h)) {
+            const cudaError_t e = cudaMemsetAsync(large_flag(h), 0, 4, s);
+            if (e != cudaSuccess) return cuda_fail(h, e, "memset");
+        }
         LFSGM_TRY(run(h, "census_all", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
-                                     h->d_sel_all, h->nviews, h->cen_pad, h->views_pad);
+                                     h->d_sel_all, h->nviews, h->cen_pad, h->views_pad, large_flag(h));
         }));
     } else if (h->n_sel_rest > 0) {
         LFSGM_TRY(run(h, "census_rest", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
-                                     h->d_sel_rest, h->n_sel_rest, h->cen_pad, h->views_pad);
+                                     h->d_sel_rest, h->n_sel_rest, h->cen_pad, h->views_pad, large_flag(h));
         }));
     }
     const cudaError_t e = cudaMemsetAsync(h->wide_count, 0, 8, s);
@@ -677,7 +698,8 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
     if (h->rows_maps) {
         LFSGM_TRY(run(h, "row_tasks", [&] {
             return launch_row_tasks(s, &h->rows, c.fine_labels, c.H, c.W, lo, cnt, (const long long *)off, h->row_tasks,
-                                    h->wide_count + 1, h->status, h->wide_list, h->wide_count);
+                                    h->wide_count + 1, h->status, h->wide_list, h->wide_count, large_flag(h),
+                                    census_only(h) ? h->marks : nullptr);
         }));
         LFSGM_TRY(run(h, "fine_cost", [&] {
             return launch_fine_cost_rows(s, &h->rows, h->views_pad, h->cen_pad, h->d_rowdesc, h->d_rowheads, h->row_tasks,
@@ -691,10 +713,21 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
                                    h->N, h->status);
         }));
     }
+    if (census_only(h) && h->rows_maps)
+        LFSGM_TRY(run(h, "fine_cost_runs", [&] {
+            return launch_census_runs(s, h->cen_pad, h->rows.P, h->rows.Wp, h->rows.Hp, h->d_ctab, c.fine_labels,
+                                      h->nviews, c.H, c.W, h->ref, h->marks, (const long long *)off, c.w_census, cost);
+        }));
+    if (census_only(h))
+        LFSGM_TRY(run(h, "fine_cost_census", [&] {
+            return launch_census_list(s, h->cen_pad, h->rows.P, h->rows.Wp, h->rows.Hp, h->d_ctab, c.fine_labels,
+                                      h->nviews, c.W, h->ref, lo, cnt, (const long long *)off, c.w_census, cost,
+                                      h->wide_list, h->wide_count, large_flag(h));
+        }));
     LFSGM_TRY(run(h, "fine_cost_wide", [&] {
         return launch_fine_cost_list(s, h->views_pad, h->cen_pad, h->rows.P, h->rows.Wp, h->rows.Hp, h->d_ltab,
                                      c.fine_labels, h->nviews, h->C, c.W, h->ref, lo, cnt, (const long long *)off,
-                                     c.w_l2, c.w_census, cost, h->wide_list, h->wide_count, h->list_ctas);
+                                     c.w_l2, c.w_census, cost, h->wide_list, h->wide_count, h->list_ctas, large_flag(h));
     }));
     return LFSGM_OK;
 }
