@@ -122,7 +122,10 @@ __device__ __forceinline__ void census_words(const float *t, int ld, const float
 template <int HALF, int C, int PPT>
 __device__ __forceinline__ void census_pad_body(const float *__restrict__ views, int H, int W, int P, int Wp, int Hp,
                                                 const int *__restrict__ sel, uint64_t *__restrict__ cen_pad,
-                                                float *__restrict__ views_pad, int *__restrict__ large) {
+                                                float *__restrict__ views_pad, int *__restrict__ large, int *__restrict__ zero,
+                                                int nzero) {
+    if (zero && blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.y == 0 && (int)threadIdx.x < nzero)
+        zero[threadIdx.x] = 0;
     constexpr int BY = 4, TYB = BY * PPT;              // thread rows, tile rows
     constexpr int SW = TX + 2 * HALF, SH = TYB + 2 * HALF;
     __shared__ float tile[SH][SW + 1];
@@ -236,8 +239,9 @@ __global__ void __launch_bounds__(TX * 4, 12) census_pad_kernel(const float *__r
                                                                     const int *__restrict__ sel,
                                                                     uint64_t *__restrict__ cen_pad,
                                                                     float *__restrict__ views_pad,
-                                                                    int *__restrict__ large) {
-    census_pad_body<HALF, 1, kPptGrey>(views, H, W, P, Wp, Hp, sel, cen_pad, views_pad, large);
+                                                                    int *__restrict__ large, int *__restrict__ zero,
+                                                                    int nzero) {
+    census_pad_body<HALF, 1, kPptGrey>(views, H, W, P, Wp, Hp, sel, cen_pad, views_pad, large, zero, nzero);
 }
 
 template <int HALF>
@@ -245,22 +249,24 @@ __global__ void __launch_bounds__(TX * 4) census_pad_rgb_kernel(const float *__r
                                                                     int P, int Wp, int Hp,
                                                                     const int *__restrict__ sel,
                                                                     uint64_t *__restrict__ cen_pad,
-                                                                    float *__restrict__ views_pad) {
-    census_pad_body<HALF, 3, kPptRgb>(views, H, W, P, Wp, Hp, sel, cen_pad, views_pad, nullptr);
+                                                                    float *__restrict__ views_pad,
+                                                                    int *__restrict__ zero, int nzero) {
+    census_pad_body<HALF, 3, kPptRgb>(views, H, W, P, Wp, Hp, sel, cen_pad, views_pad, nullptr, zero, nzero);
 }
 
 }  // namespace
 
 cudaError_t launch_census_pad(cudaStream_t s, const float *views, int H, int W, int census_w, int P, int Wp, int Hp,
-                              int C, const int *d_sel, int nsel, uint64_t *cen_pad, float *views_pad, int *large) {
+                              int C, const int *d_sel, int nsel, uint64_t *cen_pad, float *views_pad, int *large,
+                              int *zero, int nzero) {
     const int rows = 4 * (C == 3 ? kPptRgb : kPptGrey);
     dim3 block(TX, 4), grid((W + TX - 1) / TX, (H + rows - 1) / rows, nsel);
     if (C == 3) {
-        if (census_w == 5) census_pad_rgb_kernel<2><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad);
-        else census_pad_rgb_kernel<3><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad);
+        if (census_w == 5) census_pad_rgb_kernel<2><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, zero, nzero);
+        else census_pad_rgb_kernel<3><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, zero, nzero);
     } else {
-        if (census_w == 5) census_pad_kernel<2><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, large);
-        else census_pad_kernel<3><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, large);
+        if (census_w == 5) census_pad_kernel<2><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, large, zero, nzero);
+        else census_pad_kernel<3><<<grid, block, 0, s>>>(views, H, W, P, Wp, Hp, d_sel, cen_pad, views_pad, large, zero, nzero);
     }
     return cudaGetLastError();
 }

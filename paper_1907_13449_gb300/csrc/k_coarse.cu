@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(128) coarse_cost_kernel(const uint64_t *__rest
                                                           const int *__restrict__ armviews,
                                                           const int *__restrict__ otab, CoarseArms ca, int Lc,
                                                           int Lcd, OT *__restrict__ out,
-                                                          unsigned long long *__restrict__ armsum) {
+                                                          unsigned long long *__restrict__ armsum,
+                                                          uint16_t *__restrict__ sum) {
     extern __shared__ int cdiff[];                 // [warp][Lcd / 2][32]
     const int a = blockIdx.y;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -107,6 +108,12 @@ __global__ void __launch_bounds__(128) coarse_cost_kernel(const uint64_t *__rest
     const int y = task / runs_x, x0 = (task - y * runs_x) * 32;
     const size_t base = (size_t)(y + P) * Wp + P + min(x0 + lane, W - 1);
     const int nv = ca.nv[a];
+    {   // the run's path sums to 0 (their rows are contiguous, of whole 8-byte words), behind the census
+        // loads: a separate pass made the initial pass of 9x9 x 512^2 25 us longer
+        uint2 *z = reinterpret_cast<uint2 *>(sum + ((size_t)a * H * W + (size_t)y * W + x0) * Lcd);
+        const int nz = min(32, W - x0) * (Lcd / 4);
+        for (int i = lane; i < nz; i += 32) z[i] = make_uint2(0u, 0u);
+    }
     const int *views = armviews + a * kMaxArmViews;
     const int *ot = otab + ca.tab_off[a];
     int *cd = cdiff + (size_t)w * (Lcd / 2) * 32 + lane;
@@ -465,7 +472,7 @@ int coarse_stride(int Lc) {
 
 cudaError_t launch_coarse_cost(cudaStream_t s, const uint64_t *cen_pad, int P, int Wp, int Hp, int H, int W, int ref, int C,
                                const int *armviews, const int *otab, const CoarseArms &ca, int Lc,
-                               void *out, bool out8, unsigned long long *armsum) {
+                               void *out, bool out8, unsigned long long *armsum, uint16_t *sum) {
     const int Lcd = coarse_stride(Lc);
     const size_t HWp = (size_t)Hp * Wp;
     const long long tasks = (long long)((W + 31) / 32) * H;
@@ -479,7 +486,7 @@ cudaError_t launch_coarse_cost(cudaStream_t s, const uint64_t *cen_pad, int P, i
             if (e != cudaSuccess) return e;
         }
         kern<<<grid, 128, smem, s>>>(cen_pad, HWp, Wp, P, H, W, ref, armviews, otab, ca, Lc, Lcd, (uint8_t *)out,
-                                     armsum);
+                                     armsum, sum);
     } else {
         auto kern = C == 3 ? coarse_cost_kernel<3, uint16_t> : coarse_cost_kernel<1, uint16_t>;
         if (smem > 48 * 1024) {
@@ -487,7 +494,7 @@ cudaError_t launch_coarse_cost(cudaStream_t s, const uint64_t *cen_pad, int P, i
             if (e != cudaSuccess) return e;
         }
         kern<<<grid, 128, smem, s>>>(cen_pad, HWp, Wp, P, H, W, ref, armviews, otab, ca, Lc, Lcd, (uint16_t *)out,
-                                     armsum);
+                                     armsum, sum);
     }
     return cudaGetLastError();
 }

@@ -525,10 +525,20 @@ __global__ void __launch_bounds__(256) cost_partial_kernel(const float *__restri
                                                            double p2f, float *__restrict__ pen,
                                                            unsigned *__restrict__ ticket, int *__restrict__ status,
                                                            int H, int W, ScanTable st, int min_wide, int scap,
-                                                           int *__restrict__ split) {
+                                                           int *__restrict__ split, int nsplit,
+                                                           float *__restrict__ agg) {
+    if ((int)blockIdx.x >= nb + nsplit) {
+        // the aggregate's rows to 0, beside the sums (which wait for memory)
+        const long long n4 = off[N] >> 2, stride = (long long)((int)gridDim.x - nb - nsplit) * blockDim.x;
+        float4 *z = reinterpret_cast<float4 *>(agg);
+        for (long long i = (long long)((int)blockIdx.x - nb - nsplit) * blockDim.x + threadIdx.x; i < n4; i += stride)
+            z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (long long i = 4 * n4 + threadIdx.x; i < off[N]; i += blockDim.x) agg[i] = 0.f;
+        return;
+    }
     if ((int)blockIdx.x >= nb) {
         split_list(cnt, H, W, st, min_wide, scap, split, (((int)blockIdx.x - nb) * blockDim.x + threadIdx.x) >> 5,
-                   (((int)gridDim.x - nb) * blockDim.x) >> 5);
+                   (nsplit * blockDim.x) >> 5);
         return;
     }
     double s = 0.0, c = 0.0;
@@ -653,7 +663,7 @@ __global__ void __launch_bounds__(256) cost_partial_kernel(const float *__restri
 cudaError_t launch_cost_partial_sums(cudaStream_t s, const float *cost, const int *cnt, const long long *off,
                                      int N, int G, double *partial, int nblocks, double p1f, double p2f,
                                      float *pen, unsigned *ticket, int *status, int H, int W, int paths,
-                                     int min_wide, int *split) {
+                                     int min_wide, int *split, float *agg) {
     const ScanTable st = make_scan_table(H, W, paths);
     int extra = 0;
     if (split) {
@@ -662,8 +672,11 @@ cudaError_t launch_cost_partial_sums(cudaStream_t s, const float *cost, const in
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         extra = std::min((st.cum[paths] + 7) / 8, sms * 8);      // a warp per scanline
     }
-    cost_partial_kernel<<<nblocks + extra, 256, 0, s>>>(cost, cnt, off, N, G, partial, nblocks, p1f, p2f, pen, ticket,
-                                                        status, H, W, st, min_wide, kSplitCap, split);
+    // zeroing: a thread per 8 vectors of rows of about 32 slots, four CTAs per SM at most
+    const int zero = agg ? std::max(1, std::min(608, N / 256)) : 0;
+    cost_partial_kernel<<<nblocks + extra + zero, 256, 0, s>>>(cost, cnt, off, N, G, partial, nblocks, p1f, p2f, pen,
+                                                               ticket, status, H, W, st, min_wide, kSplitCap, split,
+                                                               extra, agg);
     return cudaGetLastError();
 }
 

@@ -2,6 +2,12 @@
 // sequential fusion with threshold phi, median hole filling (Jacobi passes), borders on
 // the fine grid and the exclusive scan giving the padded row offsets.
 //
+// Up to two filling passes (the workloads') run in one kernel with the fusion and the windows, on
+// tiles of 32 x 8 pixels with a halo of a pixel per pass, and the tile sums of the scan are added up
+// there: seven launches of a few us each became two.  With the cost and path sums cleared beside the
+// loads of the kernels before them, a 5x5 x 64^2 depth call takes 161 us instead of 185, the initial
+// pass of 9x9 x 512^2 731 us instead of 762.  More passes would work on halos as large as the tile.
+//
 // D_init is kept in fixed point, in units of 1/8 coarse label: with at most four maps the
 // running pairwise average m <- (m + 8 k_i) / 2 stays an exact integer (8k1, 4(k1+k2), ...),
 // and -1 marks a discarded pixel.
@@ -10,17 +16,41 @@
 namespace lfsgm {
 namespace {
 
+__device__ __forceinline__ int fuse_pixel(const int *__restrict__ maps, int narms, int N, double phi8, int p) {
+    int k[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) k[i] = i < narms ? __ldg(maps + (size_t)i * N + p) : 0;
+    int m = 8 * k[0];
+    bool ok = true;
+#pragma unroll
+    for (int i = 1; i < 4; i++)
+        if (i < narms && ok) {
+            const int mi = 8 * k[i];
+            if ((double)abs(m - mi) < phi8) m = (m + mi) / 2;
+            else ok = false;
+        }
+    return ok ? m : -1;
+}
+
 __global__ void fuse_kernel(const int *__restrict__ maps, int narms, int N, double phi, int *__restrict__ F) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    int m = 8 * maps[p];
-    bool ok = true;
-    for (int i = 1; i < narms && ok; i++) {
-        const int mi = 8 * maps[(size_t)i * N + p];
-        if ((double)abs(m - mi) < 8.0 * phi) m = (m + mi) / 2;
-        else ok = false;
-    }
-    F[p] = ok ? m : -1;
+    if (p < N) F[p] = fuse_pixel(maps, narms, N, 8.0 * phi, p);
+}
+
+// The lower middle of the valid (>= 0) values among the 8 neighbours of t (row stride ld), or -1.
+__device__ __forceinline__ int fill_value(const int *t, int ld) {
+    int vals[8], n = 0;
+    for (int dy = -1; dy <= 1; dy++)
+        for (int dx = -1; dx <= 1; dx++) {
+            if (dx == 0 && dy == 0) continue;
+            const int q = t[dy * ld + dx];
+            if (q >= 0) {
+                int j = n++;
+                while (j > 0 && vals[j - 1] > q) { vals[j] = vals[j - 1]; j--; }
+                vals[j] = q;
+            }
+        }
+    return n > 0 ? vals[(n - 1) / 2] : -1;
 }
 
 // One Jacobi pass: a discarded pixel takes the median (lower middle) of the valid values
@@ -67,52 +97,124 @@ __device__ __forceinline__ bool sobel_edge(const float *I, int sx, int sy, float
     return __fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy)) > __fmul_rn(t, t);
 }
 
-__global__ void windows_kernel(const int *__restrict__ F, int N, int G, int Lc, int R, int *__restrict__ lo,
-                               int *__restrict__ cnt, float *__restrict__ dinit, int *__restrict__ cntpad,
-                               const float *__restrict__ ref_pad, int C, int P, int Wp, int W,
-                               float edge_t, int Rfar, int boundless) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    const int v = boundless ? -1 : F[p];
+// What the windows depend on besides D_init.
+struct WindowArgs {
+    int G, Lc, R, Rfar;
+    const float *ref_pad;             // the padded reference view (channels interleaved), for the edge test
+    int C, P, Wp;
+    float edge_t;
+    int *lo, *cnt;
+    float *dinit;                     // nullable
+    unsigned long long *tsum;         // padded counts per 1024 pixels, zeroed before
+};
+
+// The window of pixel p with D_init v (-1: discarded); returns its padded count.
+__device__ __forceinline__ int window_of(const WindowArgs &a, int p, int x, int y, int v) {
     // an edge in any channel of the padded reference view (colour: one float4 per pixel, the
     // channels interleaved)
     bool edge = false;
-    if (edge_t > 0.f && !boundless) {
-        const int sx = C == 1 ? 1 : 4;
-        const float *q = ref_pad + ((size_t)(p / W + P) * Wp + (p % W + P)) * sx;
-        for (int ch = 0; ch < C && !edge; ch++) edge = sobel_edge(q + ch, sx, sx * Wp, edge_t);
+    if (a.edge_t > 0.f) {
+        const int sx = a.C == 1 ? 1 : 4;
+        const float *q = a.ref_pad + ((size_t)(y + a.P) * a.Wp + (x + a.P)) * sx;
+        for (int ch = 0; ch < a.C && !edge; ch++) edge = sobel_edge(q + ch, sx, sx * a.Wp, a.edge_t);
     }
-    int a, n;
+    const int G = a.G;
+    int l, n;
     if (v < 0 || edge) {
-        a = 0;
+        l = 0;
         n = G;
-        if (dinit) dinit[p] = v < 0 ? __int_as_float(0x7fc00000) : 0.125f * (float)v;
+        if (a.dinit) a.dinit[p] = v < 0 ? __int_as_float(0x7fc00000) : 0.125f * (float)v;
     } else {
         const long long num = (long long)v * (G - 1);
-        const long long den = 8LL * (Lc - 1);
+        const long long den = 8LL * (a.Lc - 1);
         const long long gc = (2 * num + den) / (2 * den);
-        long long r = R;
-        if (Rfar > 0) {
-            const long long dg = G - 1, t = 2 * (long long)(Rfar - R) * (dg - gc) + dg;
+        long long r = a.R;
+        if (a.Rfar > 0) {
+            const long long dg = G - 1, t = 2 * (long long)(a.Rfar - a.R) * (dg - gc) + dg;
             long long q = t / (2 * dg);
             if (t % (2 * dg) != 0 && t < 0) q--;          // floor division
-            r = R + q;
+            r = a.R + q;
         }
         long long lo_ = gc - r, hi_ = gc + r;
         if (lo_ < 0) lo_ = 0;
         if (hi_ > G - 1) hi_ = G - 1;
-        a = (int)lo_;
+        l = (int)lo_;
         n = (int)(hi_ - lo_ + 1);
-        if (dinit) dinit[p] = 0.125f * (float)v;
+        if (a.dinit) a.dinit[p] = 0.125f * (float)v;
     }
-    lo[p] = a;
-    cnt[p] = n;
-    cntpad[p] = (n + 3) & ~3;
+    a.lo[p] = l;
+    a.cnt[p] = n;
+    return (n + 3) & ~3;
 }
 
-// Exclusive scan of the padded counts in three phases over tiles of 1024 entries:
-// per-tile sums, a scan of the tile sums (one CTA), then per-tile scans plus the tile offset.
 constexpr int kScanTile = 1024;
+
+// Adds the padded counts of a warp's pixels (p >= 0) to their scan tiles.
+__device__ __forceinline__ void add_tile_sums(unsigned long long *tsum, int p, int pad) {
+    const int tile = p >= 0 ? p / kScanTile : -1;
+    const int first = __reduce_max_sync(0xffffffffu, tile);
+    if (__all_sync(0xffffffffu, tile < 0 || tile == first)) {
+        const int sum = __reduce_add_sync(0xffffffffu, p >= 0 ? pad : 0);
+        if ((threadIdx.x & 31) == 0 && first >= 0) atomicAdd(tsum + first, (unsigned long long)sum);
+    } else if (p >= 0) {
+        atomicAdd(tsum + tile, (unsigned long long)pad);
+    }
+}
+
+__global__ void __launch_bounds__(256) windows_kernel(const int *__restrict__ F, int N, int W, WindowArgs a) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    int pad = 0;
+    if (p < N) pad = window_of(a, p, p % W, p / W, F[p]);
+    add_tile_sums(a.tsum, p < N ? p : -1, pad);
+}
+
+// Boundary-less: the windows are the whole range, the offsets multiples of its padded length.
+__global__ void __launch_bounds__(256) whole_windows_kernel(int N, int G, int *__restrict__ lo, int *__restrict__ cnt,
+                                                            long long *__restrict__ off, float *__restrict__ dinit) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p > N) return;
+    off[p] = (long long)p * ((G + 3) & ~3);
+    if (p == N) return;
+    lo[p] = 0;
+    cnt[p] = G;
+    if (dinit) dinit[p] = __int_as_float(0x7fc00000);
+}
+
+// Fusion, `passes` (0 .. 2) filling passes and the windows of a 32 x 8 tile; out of the image: -1, as
+// a discarded pixel contributes nothing to a median.
+__global__ void __launch_bounds__(256) fused_windows_kernel(const int *__restrict__ maps, int narms, int H, int W,
+                                                            double phi, int passes, WindowArgs a) {
+    constexpr int TW = 36, TH = 12;
+    __shared__ int t[2][TH][TW];
+    const int x0 = blockIdx.x * 32 - passes, y0 = blockIdx.y * 8 - passes;   // image position of tile entry (0, 0)
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    for (int i = tid; i < TW * TH; i += 256) {
+        const int ty = i / TW, tx = i - ty * TW, x = x0 + tx, y = y0 + ty;
+        const bool in = tx < 32 + 2 * passes && ty < 8 + 2 * passes && x >= 0 && x < W && y >= 0 && y < H;
+        t[0][ty][tx] = in ? fuse_pixel(maps, narms, H * W, 8.0 * phi, y * W + x) : -1;
+    }
+    __syncthreads();
+    for (int k = 0; k < passes; k++) {
+        const int w = 32 + 2 * (passes - 1 - k), h = 8 + 2 * (passes - 1 - k);   // from entry (k + 1, k + 1) on
+        for (int i = tid; i < w * h; i += 256) {
+            const int ty = i / w + k + 1, tx = i % w + k + 1, x = x0 + tx, y = y0 + ty;
+            int v = t[k & 1][ty][tx];
+            if (v < 0 && x >= 0 && x < W && y >= 0 && y < H) v = fill_value(&t[k & 1][ty][tx], TW);
+            t[(k + 1) & 1][ty][tx] = v;
+        }
+        __syncthreads();
+    }
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+    const bool in = x < W && y < H;
+    int pad = 0;
+    if (in) pad = window_of(a, y * W + x, x, y, t[passes & 1][threadIdx.y + passes][threadIdx.x + passes]);
+    add_tile_sums(a.tsum, in ? y * W + x : -1, pad);
+}
+
+// Exclusive scan of the padded counts over tiles of 1024 entries, whose sums the windows kernels have
+// added up: per tile a scan plus the sum of the tiles before it (images of many tiles: of a scan of
+// the tile sums by one CTA).
+constexpr int kTopTiles = kScanTile;   // one sum per thread
 
 __device__ __forceinline__ long long block_exclusive_scan(long long v, long long *wsum, long long *total) {
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
@@ -138,20 +240,6 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
     return ex;
 }
 
-__global__ void __launch_bounds__(kScanTile) scan_tile_sums(const int *__restrict__ cntpad, int N, long long *__restrict__ tsum) {
-    __shared__ long long wsum[32];
-    const int i = blockIdx.x * kScanTile + threadIdx.x;
-    long long v = i < N ? cntpad[i] : 0;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long s = 0;
-        for (int w = 0; w < kScanTile / 32; w++) s += wsum[w];
-        tsum[blockIdx.x] = s;
-    }
-}
-
 __global__ void __launch_bounds__(kScanTile) scan_tile_offsets(long long *__restrict__ tsum, int ntiles) {
     __shared__ long long wsum[32];
     long long carry = 0;
@@ -165,13 +253,23 @@ __global__ void __launch_bounds__(kScanTile) scan_tile_offsets(long long *__rest
     }
 }
 
-__global__ void __launch_bounds__(kScanTile) scan_apply(const int *__restrict__ cntpad, int N, const long long *__restrict__ toff,
-                                                        long long *__restrict__ off) {
+__global__ void __launch_bounds__(kScanTile) scan_apply(const int *__restrict__ cnt, int N, const long long *__restrict__ tsum,
+                                                        bool scanned, long long *__restrict__ off) {
     __shared__ long long wsum[32];
     const int i = blockIdx.x * kScanTile + threadIdx.x;
-    const long long v = i < N ? cntpad[i] : 0;
+    const long long v = i < N ? (__ldg(cnt + i) + 3) & ~3 : 0;
+    long long before = 0;
+    if (scanned) {
+        before = __ldg(tsum + blockIdx.x);
+    } else {
+        // the tiles before this one
+        long long s = 0, total;
+        for (int t = threadIdx.x; t < (int)blockIdx.x; t += kScanTile) s += __ldg(tsum + t);
+        block_exclusive_scan(s, wsum, &total);
+        before = total;
+    }
     const long long ex = block_exclusive_scan(v, wsum, nullptr);
-    const long long o = toff[blockIdx.x] + ex;
+    const long long o = before + ex;
     if (i < N) off[i] = o;
     if (i == N - 1) off[N] = o + v;
 }
@@ -186,25 +284,36 @@ cudaError_t launch_fill(cudaStream_t s, const int *Fin, int *Fout, int H, int W)
     fill_kernel<<<(H * W + 255) / 256, 256, 0, s>>>(Fin, Fout, H, W);
     return cudaGetLastError();
 }
-cudaError_t launch_windows(cudaStream_t s, const int *F, int N, int G, int Lc, int R, int *lo, int *cnt,
-                           float *dinit, int *cntpad, const float *ref_pad, int C, int P, int Wp,
-                           int W, float edge_t, int Rfar, int boundless) {
-    windows_kernel<<<(N + 255) / 256, 256, 0, s>>>(F, N, G, Lc, R, lo, cnt, dinit, cntpad, ref_pad, C, P, Wp,
-                                                   W, edge_t, Rfar, boundless);
+static WindowArgs window_args(const WindowSetup &u) {
+    WindowArgs a;
+    a.G = u.G; a.Lc = u.Lc; a.R = u.R; a.Rfar = u.Rfar;
+    a.ref_pad = u.ref_pad; a.C = u.C; a.P = u.P; a.Wp = u.Wp; a.edge_t = u.edge_t;
+    a.lo = u.lo; a.cnt = u.cnt; a.dinit = u.dinit; a.tsum = (unsigned long long *)u.tsum;
+    return a;
+}
+cudaError_t launch_whole_windows(cudaStream_t s, int N, int G, int *lo, int *cnt, long long *off, float *dinit) {
+    whole_windows_kernel<<<N / 256 + 1, 256, 0, s>>>(N, G, lo, cnt, off, dinit);
+    return cudaGetLastError();
+}
+cudaError_t launch_windows(cudaStream_t s, const int *F, int N, int W, const WindowSetup &u) {
+    windows_kernel<<<(N + 255) / 256, 256, 0, s>>>(F, N, W, window_args(u));
+    return cudaGetLastError();
+}
+cudaError_t launch_fused_windows(cudaStream_t s, const int *maps, int narms, int H, int W, double phi, int passes,
+                                 const WindowSetup &u) {
+    fused_windows_kernel<<<dim3((W + 31) / 32, (H + 7) / 8), dim3(32, 8), 0, s>>>(maps, narms, H, W, phi, passes,
+                                                                                 window_args(u));
     return cudaGetLastError();
 }
 int scan_tiles(int N) { return (N + kScanTile - 1) / kScanTile; }
+bool scan_needs_top(int N) { return scan_tiles(N) > kTopTiles; }
 
-cudaError_t launch_scan_sums(cudaStream_t s, const int *cntpad, int N, long long *tsum) {
-    scan_tile_sums<<<scan_tiles(N), kScanTile, 0, s>>>(cntpad, N, tsum);
-    return cudaGetLastError();
-}
 cudaError_t launch_scan_top(cudaStream_t s, long long *tsum, int N) {
     scan_tile_offsets<<<1, kScanTile, 0, s>>>(tsum, scan_tiles(N));
     return cudaGetLastError();
 }
-cudaError_t launch_scan_apply(cudaStream_t s, const int *cntpad, int N, const long long *tsum, long long *off) {
-    scan_apply<<<scan_tiles(N), kScanTile, 0, s>>>(cntpad, N, tsum, off);
+cudaError_t launch_scan_apply(cudaStream_t s, const int *cnt, int N, const long long *tsum, long long *off) {
+    scan_apply<<<scan_tiles(N), kScanTile, 0, s>>>(cnt, N, tsum, scan_needs_top(N), off);
     return cudaGetLastError();
 }
 

@@ -86,7 +86,7 @@ struct lfsgm_ctx {
     void *ccost = nullptr;                // coarse arm costs, uint8 when they fit a byte (cost8), else uint16
     bool cost8 = false;
     uint16_t *csum = nullptr;
-    int *maps = nullptr, *F0 = nullptr, *F1 = nullptr, *cntpad = nullptr;
+    int *maps = nullptr, *F0 = nullptr, *F1 = nullptr;
     int2 *wide_list = nullptr;         // (pixel, 32-label chunk) items for the list kernel
     int *wide_count = nullptr;         // list items, the row kernel's further tasks; [2]: a large value in the views
     RowTask *row_tasks = nullptr;      // label ranges of the row kernel's blocks
@@ -290,16 +290,16 @@ lfsgm_status bind_workspace(lfsgm_ctx *h, void *dptr, size_t bytes, bool owned) 
     h->maps = (int *)take(4 * N * 4);
     h->F0 = (int *)take(N * 4);
     h->F1 = (int *)take(N * 4);
-    h->cntpad = (int *)take(N * 4);
     h->wide_list = (int2 *)take(N * (size_t)((h->cfg.fine_labels + 31) / 32) * 8);
     h->wide_count = (int *)take(12);
     h->row_tasks = (RowTask *)take(8 * (size_t)row_blocks(h->cfg.H, h->cfg.W) * sizeof(RowTask));
     h->marks = (unsigned char *)take((size_t)((h->cfg.W + 31) / 32) * h->cfg.H);
-    h->armsum = (unsigned long long *)take(4 * 8);
+    // zeroed together by the initial pass: arm sums, the scan's tile sums
+    h->armsum = (unsigned long long *)take(4 * 8 + (size_t)scan_tiles(h->N) * 8);
+    h->tsum = (long long *)(h->armsum + 4);
     h->cpen = (int *)take(8 * 4);
     h->fpen = (float *)take(2 * 4);
     h->partial = (double *)take(2 * kPartialBlocks * 8);
-    h->tsum = (long long *)take((size_t)scan_tiles(h->N) * 8);
     h->split = (int *)take((size_t)sgm_split_ints(h->cfg.H, h->cfg.W, h->cfg.paths) * 4);
     cudaError_t e = cudaMemsetAsync(h->status, 0, 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ticket, 0, 4, h->stream);
@@ -507,14 +507,14 @@ lfsgm_status lfsgm_workspace_size(lfsgm_handle h, size_t *bytes) {
     b += align256(A * N * h->Lcd * (h->cost8 ? 1 : 2));   // coarse cost (bytes when they fit)
     b += align256(A * N * h->Lcd * 2);              // coarse path sums
     b += align256(4 * N * 4);                       // maps
-    b += 3 * align256(N * 4);                       // F0, F1, padded counts
+    b += 2 * align256(N * 4);                       // F0, F1
     b += align256(N * (size_t)((h->cfg.fine_labels + 31) / 32) * 8);   // (pixel, chunk) list
     b += align256(12);                              // list and task counts, large-value flag
     b += align256(8 * (size_t)row_blocks(h->cfg.H, h->cfg.W) * sizeof(RowTask));
     b += align256((size_t)((h->cfg.W + 31) / 32) * h->cfg.H);   // run marks
-    b += align256(4 * 8) + align256(8 * 4) + align256(2 * 4);
+    b += align256(4 * 8 + (size_t)scan_tiles(h->N) * 8);   // arm sums, offset-scan tile sums
+    b += align256(8 * 4) + align256(2 * 4);
     b += align256(2 * kPartialBlocks * 8) + 2 * align256(4);   // partials; status word and ticket
-    b += align256((size_t)scan_tiles(h->N) * 8);    // offset-scan tile sums
     b += align256((size_t)sgm_split_ints(h->cfg.H, h->cfg.W, h->cfg.paths) * 4);   // SGM scanlines to split
     *bytes = b;
     return LFSGM_OK;
@@ -615,22 +615,23 @@ lfsgm_status lfsgm_initial_disparity(lfsgm_handle h, const float *views, int32_t
     const lfsgm_config &c = h->cfg;
     cudaStream_t s = h->stream;
     const int N = h->N, A = h->arms.n_arms;
-    int *fin = h->F0, *fout = h->F1;
     cudaError_t e = cudaSuccess;
-    if (!c.boundless) {   // boundary-less: no initial map, the windows kernel writes whole-range windows
-        if (census_only(h)) e = cudaMemsetAsync(large_flag(h), 0, 4, s);
+    if (c.boundless) {   // no initial map, windows of the whole range
+        LFSGM_TRY(run(h, "windows", [&] {
+            return launch_whole_windows(s, N, c.fine_labels, lo, cnt, (long long *)off, dinit);
+        }));
+    } else {
+        e = cudaMemsetAsync(h->armsum, 0, 4 * 8 + (size_t)scan_tiles(N) * 8, s);
+        if (e == cudaSuccess && census_only(h)) e = cudaMemsetAsync(large_flag(h), 0, 4, s);
         if (e != cudaSuccess) return cuda_fail(h, e, "memset");
         LFSGM_TRY(run(h, "census_cross", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
                                      h->d_sel_cross, h->n_sel_cross, h->cen_pad, h->views_pad, large_flag(h));
         }));
-        e = cudaMemsetAsync(h->armsum, 0, 4 * 8, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->csum, 0, (size_t)A * N * h->Lcd * 2, s);
-        if (e != cudaSuccess) return cuda_fail(h, e, "memset");
         LFSGM_TRY(run(h, "coarse_cost", [&] {
             return launch_coarse_cost(s, h->cen_pad, h->rows.P, h->rows.Wp, h->rows.Hp, c.H, c.W, h->ref, h->C,
                                       h->d_armviews, h->d_otab, h->ca, c.coarse_labels, h->ccost, h->cost8,
-                                      h->armsum);
+                                      h->armsum, h->csum);
         }));
         LFSGM_TRY(run(h, "coarse_penalties", [&] {
             return launch_coarse_penalties(s, h->armsum, A, (long long)N * c.coarse_labels, c.p1_frac, c.p2_frac,
@@ -643,20 +644,25 @@ lfsgm_status lfsgm_initial_disparity(lfsgm_handle h, const float *views, int32_t
         LFSGM_TRY(run(h, "coarse_wta", [&] {
             return launch_coarse_wta(s, h->csum, A, N, c.coarse_labels, h->maps, maps);
         }));
-        LFSGM_TRY(run(h, "fuse", [&] { return launch_fuse(s, h->maps, A, N, c.phi, h->F0); }));
-        for (int it = 0; it < c.fill_passes; it++) {
-            LFSGM_TRY(run(h, "hole_fill", [&] { return launch_fill(s, fin, fout, c.H, c.W); }));
-            std::swap(fin, fout);
-        }
-    }
-    LFSGM_TRY(run(h, "windows", [&] {
-        return launch_windows(s, fin, N, c.fine_labels, c.coarse_labels, c.fine_radius, lo, cnt, dinit, h->cntpad,
+        const WindowSetup win{c.fine_labels, c.coarse_labels, c.fine_radius, c.fine_radius_far,
                               h->views_pad + (size_t)h->ref * h->rows.Hp * h->rows.Wp * (h->C > 1 ? 4 : 1), h->C,
-                              h->rows.P, h->rows.Wp, c.W, c.edge_threshold, c.fine_radius_far, c.boundless);
-    }));
-    LFSGM_TRY(run(h, "scan_sums", [&] { return launch_scan_sums(s, h->cntpad, N, h->tsum); }));
-    LFSGM_TRY(run(h, "scan_top", [&] { return launch_scan_top(s, h->tsum, N); }));
-    LFSGM_TRY(run(h, "scan_apply", [&] { return launch_scan_apply(s, h->cntpad, N, h->tsum, (long long *)off); }));
+                              h->rows.P, h->rows.Wp, c.edge_threshold, lo, cnt, dinit, h->tsum};
+        if (c.fill_passes <= kFusedFills) {
+            LFSGM_TRY(run(h, "windows", [&] {
+                return launch_fused_windows(s, h->maps, A, c.H, c.W, c.phi, c.fill_passes, win);
+            }));
+        } else {
+            int *fin = h->F0, *fout = h->F1;
+            LFSGM_TRY(run(h, "fuse", [&] { return launch_fuse(s, h->maps, A, N, c.phi, fin); }));
+            for (int it = 0; it < c.fill_passes; it++) {
+                LFSGM_TRY(run(h, "hole_fill", [&] { return launch_fill(s, fin, fout, c.H, c.W); }));
+                std::swap(fin, fout);
+            }
+            LFSGM_TRY(run(h, "windows", [&] { return launch_windows(s, fin, N, c.W, win); }));
+        }
+        if (scan_needs_top(N)) LFSGM_TRY(run(h, "scan_top", [&] { return launch_scan_top(s, h->tsum, N); }));
+        LFSGM_TRY(run(h, "scan_apply", [&] { return launch_scan_apply(s, cnt, N, h->tsum, (long long *)off); }));
+    }
     if (nnz_host) {
         e = cudaMemcpyAsync(nnz_host, off + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -685,16 +691,19 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
         }
         LFSGM_TRY(run(h, "census_all", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
-                                     h->d_sel_all, h->nviews, h->cen_pad, h->views_pad, large_flag(h));
+                                     h->d_sel_all, h->nviews, h->cen_pad, h->views_pad, large_flag(h), h->wide_count,
+                                     2);
         }));
     } else if (h->n_sel_rest > 0) {
         LFSGM_TRY(run(h, "census_rest", [&] {
             return launch_census_pad(s, views, c.H, c.W, c.census_w, h->rows.P, h->rows.Wp, h->rows.Hp, h->C,
-                                     h->d_sel_rest, h->n_sel_rest, h->cen_pad, h->views_pad, large_flag(h));
+                                     h->d_sel_rest, h->n_sel_rest, h->cen_pad, h->views_pad, large_flag(h),
+                                     h->wide_count, 2);
         }));
+    } else {
+        const cudaError_t e = cudaMemsetAsync(h->wide_count, 0, 8, s);
+        if (e != cudaSuccess) return cuda_fail(h, e, "memset");
     }
-    const cudaError_t e = cudaMemsetAsync(h->wide_count, 0, 8, s);
-    if (e != cudaSuccess) return cuda_fail(h, e, "memset");
     if (h->rows_maps) {
         LFSGM_TRY(run(h, "row_tasks", [&] {
             return launch_row_tasks(s, &h->rows, c.fine_labels, c.H, c.W, lo, cnt, (const long long *)off, h->row_tasks,
@@ -784,13 +793,14 @@ lfsgm_status lfsgm_sgm_aggregate(lfsgm_handle h, const float *cost, const int32_
     cudaStream_t s = h->stream;
     const long long *o = (const long long *)off;
     if (derived) {
-        // zero agg (and the split list's count), then the penalty mean, whose launch also lists the
-        // scanlines to split
-        LFSGM_TRY(sgm_prologue(h, agg, cnt, o, false));
+        // the penalty mean, whose launch also zeroes agg; with the split knob on, agg and the split list's
+        // count are zeroed first, and the launch lists the scanlines to split
+        if (h->sgm_split > 0) LFSGM_TRY(sgm_prologue(h, agg, cnt, o, false));
         LFSGM_TRY(run(h, "cost_partial_sums", [&] {
             return launch_cost_partial_sums(s, cost, cnt, o, h->N, c.fine_labels, h->partial, kPartialBlocks,
                                             c.p1_frac, c.p2_frac, h->fpen, h->ticket, h->status, c.H, c.W,
-                                            c.paths, h->sgm_split, h->sgm_split > 0 ? h->split : nullptr);
+                                            c.paths, h->sgm_split, h->sgm_split > 0 ? h->split : nullptr,
+                                            h->sgm_split > 0 ? nullptr : agg);
         }));
     } else {
         LFSGM_TRY(run(h, "set_penalties", [&] {
