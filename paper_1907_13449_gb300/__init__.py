@@ -404,7 +404,8 @@ def lfsgm_set_sgm_warps(h, warps_per_cta=0):
 
 def lfsgm_set_sgm_split(h, min_wide=0):
     """Speed knob of the fine SGM: scanlines crossing at least min_wide windows wider than 32
-    labels run on all warps of a CTA (0: none)."""
+    labels run on all warps of a CTA (0: 24 for images of 256 pixels or more in a direction, unless
+    every window is the whole range; a large value: none)."""
     _check(load().lfsgm_set_sgm_split(h, int(min_wide)), h)
 
 

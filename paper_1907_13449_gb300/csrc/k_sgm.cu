@@ -16,9 +16,16 @@
 // concurrently and add into agg (zeroed by the caller) with float atomics.  A run of equal windows of
 // 33 to 128 labels (whole-range searches) keeps the predecessor's row in registers, four consecutive
 // labels a lane: one vector load and one vector reduction a step, the neighbours across lanes by two
-// shuffles (7x1 x 555x650, 121 labels: 295 instructions a step in shared-memory chunks, 956 us).  Optionally the few
-// scanlines that cross many wide windows (a speed knob) run on all the warps of a CTA each, which
-// share the wide steps' chunks (sgm_scanline SPLIT); a small kernel lists them first.
+// shuffles (7x1 x 555x650, 121 labels: 295 instructions a step in shared-memory chunks, 956 us).  The few
+// scanlines that cross many wide windows (a speed knob's threshold) run on all the warps of a CTA each, which
+// share the wide steps (sgm_scanline SPLIT); the kernel before lists them.  Where few windows are wide, a warp
+// takes two scanlines (sgm_pair).
+//
+// What bounds it: issue slots while all scanlines run (72 instructions a narrow step, 100 for two in
+// sgm_pair), then the scanlines with the most wide steps, and L2 latency where there are few scanlines.
+// fine_sgm of 9x9 x 512^2 (31 labels, 0.8 % wide): 297 us before the split by default and the pairs, 209 now
+// (recording, not paired: 382 and 314); 15x15 x 434 x 625 (no wide windows): 182 and 165; 4x4 x 720 x 1280, 16
+// directions, 17 labels: 1163 and 800.
 //
 // Reproducible sum over the directions.  The aggregate C_s(p,g) = sum_r L_r(p,g) must not depend on
 // the order in which the directions' atomics arrive.  Every exact L_r(p,g) lies in [0, B] with
@@ -39,6 +46,9 @@ namespace lfsgm {
 namespace {
 
 constexpr int kSgmWarps = 4;      // default warps (scanlines) per CTA; 2, 4 or 8 (a speed knob)
+constexpr int kSplitRing = 4;     // cost rows of a split scanline's wide steps on their way (a power of two)
+constexpr int kPairFrom = 1024;   // scanlines from which on a warp may take two (twelve 5x5 x 251 x 283 side by side:
+                                  // 2015 us with one, 1914 with two; 764 scanlines of 5x5 x 64^2: 20.6 and 21.0)
 constexpr int kSplitCap = 256;    // most scanlines split across a CTA's warps (more qualify: none is)
 
 // L rounded to a multiple of q (see above); B = C + P2 of the cell.  With M = 1.5 x 2^(floor(log2 B)
@@ -50,23 +60,86 @@ __device__ __forceinline__ float det_addend(float L, float B, int mk) {
     return __fsub_rn(__fadd_rn(fminf(L, B), M), M);
 }
 
+// agg[0 .. n) to 0 by `stride` threads, this one the i0-th (agg 16-byte aligned).
+__device__ __forceinline__ void zero_rows(float *agg, long long n, long long i0, long long stride) {
+    const long long n4 = n >> 2;
+    float4 *z = reinterpret_cast<float4 *>(agg);
+    for (long long i = i0; i < n4; i += stride) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i0 < (n & 3)) agg[4 * n4 + i0] = 0.f;
+}
+
 __device__ __forceinline__ float warp_min(float v) {
     float r;
     asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 
+// st.cum[r] by selects (a run-time index would copy the table to the stack).
+__device__ __forceinline__ int scan_base(const ScanTable &st, int r) {
+    int base = 0;
+#pragma unroll
+    for (int q = 1; q < kMaxPaths; q++)
+        if (q <= r) base = st.cum[q];
+    return base;
+}
+
+// Four consecutive labels j0 .. j0 + 3 of a wide step on the predecessor's row A by slot (window (pl, pn),
+// minimum m; pn = 0: the path starts; same: the windows are equal) with costs c4: the path costs into row
+// B (+inf from slot n on) and, rounded, into agg; branches into code; the running minimum and its lowest
+// slot (REC) into lmin, lslot.
+template <bool REC>
+__device__ __forceinline__ void wide_cells(float4 c4, int j0, int n, int l, int pl, int pn, bool same, unsigned top,
+                                           const float *A, float m, float P1, float P2, int mk, float *agg,
+                                           unsigned char *code, float &lmin, int &lslot, float *B) {
+    const float INF = __int_as_float(0x7f800000);
+    const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+    float v[6], L4[4], a4[4];                  // v: the predecessor's labels -1 .. 4 from j0 on
+    unsigned cd = 0u;
+    if (same) {
+        const float4 f = *reinterpret_cast<const float4 *>(A + j0);
+        v[0] = A[j0 - 1];
+        v[1] = f.x;
+        v[2] = f.y;
+        v[3] = f.z;
+        v[4] = f.w;
+        v[5] = A[j0 + 4];
+    } else {
+        // slot s is read at A[s] with s + 1 clamped (unsigned) to pn + 1: any slot outside [0, pn) lands on
+        // a sentinel (+inf), so an absent label drops out of the minimum
+#pragma unroll
+        for (int u = 0; u < 6; u++) v[u] = A[(int)min((unsigned)(l + j0 + u - pl), top) - 1];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const bool on = j0 + u < n;
+        const float t = fminf(fminf(m + P2, v[u + 1]), fminf(v[u], v[u + 2]) + P1);
+        const float Ln = pn != 0 ? c[u] + (t - m) : c[u];
+        if (REC) {
+            cd |= (pn == 0 ? 4u : (t == m + P2 ? 3u : (t == v[u + 1] ? 0u : (t == v[u] + P1 ? 1u : 2u)))) << (8 * u);
+            if (on && Ln < lmin) lslot = j0 + u;   // ascending: the lane's first minimum
+        }
+        a4[u] = on ? det_addend(Ln, c[u] + P2, mk) : 0.f;
+        L4[u] = on ? Ln : INF;
+        lmin = fminf(lmin, L4[u]);
+    }
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
+                 ::"l"(agg + j0), "f"(a4[0]), "f"(a4[1]), "f"(a4[2]), "f"(a4[3]) : "memory");
+    if (REC) *reinterpret_cast<unsigned *>(code + j0) = cd;   // the padding slots' codes are never read
+    *reinterpret_cast<float4 *>(B + j0) = make_float4(L4[0], L4[1], L4[2], L4[3]);
+}
+
 // One scanline of direction r = rs & 15, number s = rs >> 4.  NW = 1: one warp, its own rows by
 // slot (bufA, bufB) and metadata ring.  SPLIT (NW = the CTA's warps): the CTA's warps share the
 // rows; warp 0 alone runs the narrow steps (the predecessor row in its registers), and every
 // general step (a window or predecessor wider than 32 labels, or an invalid window) is spread over
-// the warps by 32-slot chunk (warp w takes chunks w, w + NW, ...), the predecessor minimum taken
+// the warps, four consecutive labels a thread (vectors of cost, aggregate and row; the next step's
+// cost one step ahead), the predecessor minimum taken
 // over the warps' minima through xm ([2][NW] minima, [2][NW] slots for REC, then the minimum that
 // warp 0 hands over after narrow steps), with one CTA barrier per general step (two after narrow
 // steps).  Every cell gets the same value either way.
 // REC: also record, for the adjoint, each cell's winning branch (0 same label, 1 label-1, 2 label+1,
 // 3 m+P2, 4 path start; the first of P2, same, g-1, g+1 that equals the minimum, as the adjoint's
-// own recurrence decides it) in codes[r * nnz_cap + slot] and each pixel's lowest minimising slot
+// own recurrence decides it) in codes[r * nnz_cap + slot] (nnz_cap a multiple of 4: vectors of codes) and each pixel's lowest minimising slot
 // in amin[r * N + p].
 template <bool REC, bool SPLIT, int NW>
 __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, const int *__restrict__ lo,
@@ -75,7 +148,7 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                                              int *__restrict__ status, int rs, int mk,
                                              unsigned char *__restrict__ codes, int *__restrict__ amin,
                                              size_t nnz_cap, float *bufA, float *bufB, int2 *meta, float *xm,
-                                             int wib) {
+                                             int wib, float *cring = nullptr, int cstride = 0) {
     const int lane = threadIdx.x & 31;
     const int r = rs & 15, s = rs >> 4;
     const int dx = dir_dx(r), dy = dir_dy(r);
@@ -100,11 +173,11 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
         if (k < len) {
             const long long p = p0 + (long long)k * dpix;
             const int l_ = __ldg(lo + p), n_ = __ldg(cnt + p);
-            const long long o_ = __ldg(off + p);
-            if (window_ok(l_, n_, G, __ldg(off + p + 1) - o_, status) && (o_ & 3) == 0 && (o_ >> 2) < 0x7fffffff) {
+            const long long o_ = __ldg(off + p), e_ = __ldg(off + p + 1);   // both multiples of 4: rows end there too
+            if (window_ok(l_, n_, G, e_ - o_, status) && ((o_ | e_) & 3) == 0 && (o_ >> 2) < 0x7fffffff) {
                 mw = l_ | (n_ << 16);
                 mo = (int)(o_ >> 2);
-            } else if ((o_ & 3) != 0 && status) {
+            } else if (((o_ | e_) & 3) != 0 && status) {
                 atomicExch(status, 7);
             }
         }
@@ -120,6 +193,7 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
     float prev = INF, m = 0.f;                 // predecessor row (one slot per lane) and its minimum
     bool in_smem = false;                      // the predecessor row is in bufA (after a general step)
     int gpar = 0;                              // SPLIT: which half of xm this general step uses
+    int asked = 0;                             // SPLIT: the wide steps before this one are requested (see below)
     int k = 0;
     // the block of metadata after the one that ends at step k (a multiple of 32)
     auto next_block = [&]() {
@@ -294,12 +368,36 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                 const long long o = 4ll * ofs;
                 float lmin = INF;
                 int lslot = 0x7fffffff;
+                if constexpr (SPLIT) {
+                    // four consecutive labels a thread; the first vectors of the wide steps up to
+                    // kSplitRing - 1 ahead are on their way to the thread's place in the cost rows
+                    const int t0 = 4 * (32 * wib + lane);
+                    if (asked < k) asked = k;
+                    for (; asked < k + kSplitRing; asked++) {
+                        const int2 w = meta[asked & 63];
+                        if ((w.x >> 16) > 32 && t0 < (w.x >> 16))
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                                         ::"r"((unsigned)__cvta_generic_to_shared(cring + (asked & (kSplitRing - 1)) * cstride + t0)),
+                                         "l"(cost + 4ll * w.y + t0) : "memory");
+                        asm volatile("cp.async.commit_group;" ::: "memory");
+                    }
+                    asm volatile("cp.async.wait_group %0;" ::"n"(kSplitRing - 1) : "memory");
+                    const bool same = l == plo && n == pn;
+                    const unsigned top = (unsigned)pn + 1u;
+                    for (int j0 = t0; j0 < n; j0 += 128 * NW) {
+                        const float4 c4 = j0 == t0 && n > 32
+                                              ? *reinterpret_cast<const float4 *>(cring + (k & (kSplitRing - 1)) * cstride + t0)
+                                              : __ldg(reinterpret_cast<const float4 *>(cost + o + j0));
+                        wide_cells<REC>(c4, j0, n, l, plo, pn, same, top, bufA, m, P1, P2, mk, agg + o,
+                                        REC ? code + o : nullptr, lmin, lslot, bufB);
+                    }
+                }
                 // sixteen of this warp's 32-label chunks per round: their cost loads are in flight
                 // together, and every chunk reads the predecessor row before any chunk stores its own
                 // (the compiler cannot tell bufA from bufB, so a store between them would order the
                 // chunks one after another)
-                constexpr int CS = 32 * NW;            // slot stride between a warp's chunks
-                for (int j0 = 32 * (SPLIT ? wib : 0) + lane; j0 < n; j0 += 16 * CS) {
+                constexpr int CS = 32;                 // slot stride between the chunks
+                for (int j0 = lane; !SPLIT && j0 < n; j0 += 16 * CS) {
                     float cc[16];
 #pragma unroll
                     for (int u = 0; u < 16; u++) cc[u] = j0 + CS * u < n ? __ldg(cost + o + j0 + CS * u) : 0.f;
@@ -399,10 +497,232 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
     }
 }
 
+// Two scanlines per warp, sixteen lanes each (half h = lane >> 4), in step: lane i of a half owns slots
+// 2i and 2i + 1 of its window (vector loads and reductions).  A narrow step takes about 100 instructions
+// for both scanlines instead of 72 for each.  A block of 32 steps is looked over once: the steps that are
+// not narrow in both halves (a path start, a window or predecessor wider than 32 labels, an invalid
+// window) are taken one by one, and those at which neither window moves need no alignment.
+// Wide steps run on the whole warp, first the one half's, then the other's, on rows by slot in shared
+// memory (row: the warp's three rows of rstride floats, the halves' and a spare one; slot -1 and slot n hold
+// +inf).
+// mt: the halves' metadata rings, 64 steps each (as in sgm_scanline).
+__device__ __forceinline__ void sgm_pair(const float *__restrict__ cost, const int *__restrict__ lo,
+                                         const int *__restrict__ cnt, const long long *__restrict__ off, int H, int W,
+                                         float P1, float P2, int G, float *__restrict__ agg, int *__restrict__ status,
+                                         int rs, bool have, int mk, float *row, int rstride, int2 *ring) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, i = lane & 15, h = lane >> 4;
+    const float INF = __int_as_float(0x7f800000);
+    const int r = rs & 15;
+    int dx, dy, x0, y0;
+    dir_of(r, dx, dy);
+    scan_start_d(dx, dy, rs >> 4, H, W, x0, y0);
+    const int len = have ? scan_steps(x0, y0, dx, dy, H, W) : 0;
+    const int p0 = y0 * W + x0, dpix = dy * W + dx;
+    const int maxlen = max(__shfl_sync(ALL, len, 0), __shfl_sync(ALL, len, 16));
+    int2 *mt = ring + 64 * h;
+    if (lane < 3) row[lane * rstride - 1] = INF;
+    // the window metadata of steps kb .. kb + 31 into the half's ring (see sgm_scanline)
+    auto fetch = [&](int kb) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = kb + 16 * u + i;
+            int2 v = make_int2(0, 0);
+            if (k < len) {
+                const int p = p0 + k * dpix;
+                const int l_ = __ldg(lo + p), n_ = __ldg(cnt + p);
+                const long long o_ = __ldg(off + p), e_ = __ldg(off + p + 1);
+                if (window_ok(l_, n_, G, e_ - o_, status) && ((o_ | e_) & 3) == 0 && (o_ >> 2) < 0x7fffffff)
+                    v = make_int2(l_ | (n_ << 16), (int)(o_ >> 2));
+                else if (((o_ | e_) & 3) != 0 && status)
+                    atomicExch(status, 7);
+            }
+            mt[k & 63] = v;
+        }
+    };
+    fetch(0);
+    __syncwarp();
+    int plo = 0, pn = 0;                          // the half's predecessor window; pn = 0: the path (re)starts
+    float v0 = INF, v1 = INF, m = 0.f;            // its slots 2i and 2i + 1 and its minimum
+    int in_smem = 0, own = h;                     // its row is (also) in shared memory, in row `own`
+    int spare = 2;                                // the row that neither half uses
+    const float2 none = make_float2(0.f, 0.f);
+    const float *cbase = cost + 2 * i;
+    float *abase = agg + 2 * i;
+    auto cost_of = [&](int2 w) {
+        return 2 * i < (w.x >> 16) ? __ldg(reinterpret_cast<const float2 *>(cbase + 4ll * w.y)) : none;
+    };
+    // slots s - 1 .. s + 2 of the predecessor row for s = 2i + d, +inf outside [0, 32) (and from pn on)
+    auto shifted = [&](int d, float &a, float &b, float &c, float &e) {
+        const int q = i + (d >> 1), odd = d & 1, s = 2 * i + d;
+        const float B = __shfl_sync(ALL, v0, q, 16), C = __shfl_sync(ALL, v1, q, 16);
+        const float D = __shfl_sync(ALL, v0, q + 1, 16), X = __shfl_sync(ALL, v1, q - 1 + 2 * odd, 16);
+        a = (unsigned)(s - 1) < 32u ? (odd ? B : X) : INF;
+        b = (unsigned)s < 32u ? (odd ? C : B) : INF;
+        c = (unsigned)(s + 1) < 32u ? (odd ? D : C) : INF;
+        e = (unsigned)(s + 2) < 32u ? (odd ? X : D) : INF;
+    };
+    // the step on the neighbours a (slot - 1), b, c (the two slots) and e; writes the cells of halves with
+    // `on`; returns the new row
+    auto cells = [&](float2 cs, int n, int ofs, float a, float b, float c, float e, bool start, bool on, float &n0,
+                     float &n1) {
+        const float q = m + P2;
+        const float t0 = fminf(fminf(q, fminf(a, c) + P1), b), t1 = fminf(fminf(q, fminf(b, e) + P1), c);
+        float L0 = cs.x + (t0 - m), L1 = cs.y + (t1 - m);
+        if (start) {
+            L0 = cs.x;
+            L1 = cs.y;
+        }
+        const bool h0 = on && 2 * i < n, h1 = on && 2 * i + 1 < n;
+        if (h0) {
+            const float s0 = det_addend(L0, cs.x + P2, mk), s1 = h1 ? det_addend(L1, cs.y + P2, mk) : 0.f;
+            asm volatile("red.global.add.v2.f32 [%0], {%1, %2};"
+                         ::"l"(abase + 4ll * ofs), "f"(s0), "f"(s1) : "memory");
+        }
+        n0 = h0 ? L0 : INF;
+        n1 = h1 ? L1 : INF;
+    };
+    auto half_min = [&](float x) {
+        const float ma = warp_min(h ? INF : x), mb = warp_min(h ? x : INF);
+        return h ? mb : ma;
+    };
+    for (int kb = 0; kb < maxlen; kb += 32) {
+        const int kbend = min(kb + 32, maxlen);
+        // the block's steps that are not narrow in both halves, and those at which neither window moves
+        unsigned special = 0u, still = 0u;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = kb + 16 * u + i;
+            const int w = mt[k & 63].x, pw = k > 0 ? mt[(k - 1) & 63].x : 0;
+            const int n = w >> 16, q = pw >> 16;
+            const unsigned sp = __ballot_sync(ALL, k < len && ((unsigned)(n - 1) >= 32u || (unsigned)(q - 1) >= 32u));
+            const unsigned mv = __ballot_sync(ALL, k < len && (w & 0xffff) != (pw & 0xffff));
+            special |= ((sp | sp >> 16) & 0xffffu) << (16 * u);
+            still |= (~(mv | mv >> 16) & 0xffffu) << (16 * u);
+        }
+        __syncwarp();                             // step kb - 1 is read; the next block takes its slots
+        fetch(kb + 32);
+        __syncwarp();
+        int k = kb;
+        while (k < kbend) {
+            const unsigned ahead = special >> (k - kb);
+            const int kend = ahead ? k + __ffs(ahead) - 1 : kbend;
+            if (k < kend) {
+                // a step on (w, c); (wn, cn) take the metadata and cost row of two steps ahead.  Three register
+                // sets in turn, and the cells in both branches: rotating one set took 20 moves a step.
+                auto step = [&](const int2 w, const float2 c, int2 &wn, float2 &cn) {
+                    wn = mt[(k + 2) & 63];
+                    cn = cost_of(wn);
+                    const int l = w.x & 0xffff, n = w.x >> 16;
+                    if (still >> (k - kb) & 1u) {
+                        float a = __shfl_up_sync(ALL, v1, 1, 16), e = __shfl_down_sync(ALL, v0, 1, 16);
+                        a = i == 0 ? INF : a;
+                        e = i == 15 ? INF : e;
+                        cells(c, n, w.y, a, v0, v1, e, false, true, v0, v1);
+                    } else {
+                        float a, b, cc, e;
+                        shifted(l - plo, a, b, cc, e);
+                        cells(c, n, w.y, a, b, cc, e, false, true, v0, v1);
+                        plo = l;
+                    }
+                    m = half_min(fminf(v0, v1));
+                    return ++k == kend;
+                };
+                int2 wa = mt[k & 63], wb = mt[(k + 1) & 63], wc;
+                float2 ca = cost_of(wa), cb = cost_of(wb), cc;
+                for (;;) {
+                    if (step(wa, ca, wc, cc)) break;
+                    if (step(wb, cb, wa, ca)) break;
+                    if (step(wc, cc, wb, cb)) break;
+                }
+                plo = mt[(k - 1) & 63].x & 0xffff;
+                pn = mt[(k - 1) & 63].x >> 16;
+                in_smem = 0;
+            }
+            if (k >= kbend) break;
+            // a step that is not narrow in both halves: the half that is, if one is, first
+            const int2 w = mt[k & 63];
+            const int l = w.x & 0xffff, n = w.x >> 16;
+            const bool gen = k < len && (n == 0 || n > 32 || pn > 32), nar = k < len && !gen;
+            {
+                float a, b, c, e, n0, n1;
+                shifted(l - plo, a, b, c, e);
+                cells(nar ? cost_of(w) : none, n, w.y, a, b, c, e, pn == 0, nar, n0, n1);
+                const float mn = half_min(fminf(n0, n1));
+                if (nar) {
+                    v0 = n0;
+                    v1 = n1;
+                    m = mn;
+                    plo = l;
+                    pn = n;
+                    in_smem = 0;
+                }
+            }
+#pragma unroll 1
+            for (int hh = 0; hh < 2; hh++) {
+                const int src = 16 * hh;
+                if (!__shfl_sync(ALL, (int)gen, src)) continue;
+                const int gn = __shfl_sync(ALL, n, src), gl = __shfl_sync(ALL, l, src);
+                if (gn == 0) {
+                    if (h == hh) pn = 0;
+                    continue;
+                }
+                const int gpn = __shfl_sync(ALL, pn, src), gpl = __shfl_sync(ALL, plo, src);
+                const int ga = __shfl_sync(ALL, own, src);
+                const float gm = __shfl_sync(ALL, m, src);
+                const long long o = 4ll * __shfl_sync(ALL, w.y, src);
+                float *A = row + ga * rstride, *B = row + spare * rstride;
+                if (h == hh && pn != 0 && !in_smem) {      // the narrow steps' last row
+                    if (2 * i < pn) A[2 * i] = v0;
+                    if (2 * i + 1 < pn) A[2 * i + 1] = v1;
+                    if (i == 0) A[pn] = INF;
+                }
+                __syncwarp();
+                float lmin = INF;
+                int lslot = 0x7fffffff;
+                const bool same = gl == gpl && gn == gpn;
+                const unsigned top = (unsigned)gpn + 1u;
+                for (int jr = 4 * lane; jr < gn; jr += 256) {
+                    float4 c4[2];                          // two vectors' loads in flight together
+#pragma unroll
+                    for (int u = 0; u < 2; u++)
+                        c4[u] = jr + 128 * u < gn ? __ldg(reinterpret_cast<const float4 *>(cost + o + jr + 128 * u))
+                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int u = 0; u < 2; u++)
+                        if (jr + 128 * u < gn)
+                            wide_cells<false>(c4[u], jr + 128 * u, gn, gl, gpl, gpn, same, top, A, gm, P1, P2, mk, agg + o,
+                                            nullptr, lmin, lslot, B);
+                }
+                const float mn = warp_min(lmin);
+                if (lane == 0) B[gn] = INF;
+                __syncwarp();
+                if (h == hh) {
+                    m = mn;
+                    own = spare;
+                    plo = gl;
+                    pn = gn;
+                    in_smem = 1;
+                    v0 = 2 * i < gn ? B[2 * i] : INF;      // for a following narrow step
+                    v1 = 2 * i + 1 < gn ? B[2 * i + 1] : INF;
+                }
+                spare = ga;
+                __syncwarp();
+            }
+            k++;
+        }
+        __syncwarp();
+    }
+}
+
 // One warp per scanline, WPC warps per CTA; with split (not null), the first scap CTAs take one
 // listed scanline each with all their warps (sgm_scanline SPLIT), and the other warps skip the
-// listed ones.  split: [0] scanlines listed, [1 .. scap] the list (rs), then a mark per scanline
-// (sgm_split_kernel); more than scap listed: none is split.
+// listed ones.  split: [0] scanlines listed, [1 .. scap] the list (rs), then the wide windows of each
+// scanline and, last, of the image (count_wide); more than scap listed: none is split.  PAIR: where the
+// image has at most pair_wide (1 %) wide windows, a warp takes two scanlines (sgm_pair), and the CTAs past
+// them have nothing to do: 512^2 pixels without wide windows 174 -> 143 us, 4x4 x 720 x 1280 with 16
+// directions and 0.6 % of them 1163 -> 800 us, but with 2 % of them 212 -> 221 us and with 10 % 321 -> 425 us,
+// since both scanlines wait for the wide steps of either.
 // Resident CTAs per SM that the register budget must allow: what the one-warp path reaches on its
 // own (72 registers without the record, 96 with it; 8 warps: 80 and 128), so that the split path
 // (more registers) does not lower the occupancy of every CTA.
@@ -410,7 +730,14 @@ __host__ __device__ constexpr int sgm_min_ctas(bool rec, int wpc) {
     return rec ? (wpc == 2 ? 10 : wpc == 4 ? 5 : 2) : (wpc == 2 ? 14 : wpc == 4 ? 7 : 3);
 }
 
-template <bool REC, int WPC>
+// Floats of the rows of fine_sgm_kernel's CTA: two per warp (PAIR: three, with room for alignment), or what a
+// split scanline takes (sgm_scanline).
+__host__ __device__ constexpr int row_floats(int wpc, int Gs, bool split, bool pair) {
+    const int own = pair ? wpc * 3 * (Gs + 8) : wpc * 2 * (Gs + 2), across = split ? 4 + (2 + kSplitRing) * (Gs + 8) : 0;
+    return own > across ? own : across;
+}
+
+template <bool REC, int WPC, bool PAIR>
 __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_kernel(const float *__restrict__ cost,
                                                                   const int *__restrict__ lo,
                                                                   const int *__restrict__ cnt,
@@ -422,90 +749,88 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
                                                                   const int *__restrict__ order, int mk,
                                                                   unsigned char *__restrict__ codes,
                                                                   int *__restrict__ amin, size_t nnz_cap,
-                                                                  const int *__restrict__ split, int scap) {
-    extern __shared__ float sm[];
+                                                                  const int *__restrict__ split, int scap,
+                                                                  int min_wide, int pair_wide) {
+    extern __shared__ __align__(16) float sm[];
     const int wib = threadIdx.x >> 5;
     // rows by slot with one sentinel slot on each side (slot -1 and slot n hold +inf), Gs + 2 floats,
     // two per warp; then per warp a ring of the metadata of this block of 32 steps and the next one,
     // by step mod 64 (read by the narrow steps with one broadcast load); then xm (SPLIT)
-    int2 *meta = reinterpret_cast<int2 *>(sm + (size_t)WPC * 2 * (Gs + 2)) + wib * 64;
-    float *xm = sm + (size_t)WPC * 2 * (Gs + 2) + WPC * 128;
+    const int rows = row_floats(WPC, Gs, split != nullptr, PAIR);
+    int2 *ring = reinterpret_cast<int2 *>(sm + rows), *meta = ring + wib * 64;
+    float *xm = sm + rows + (PAIR ? 2 : 1) * WPC * 128;
     const float P1 = __ldg(pen), P2 = __ldg(pen + 1);
     const int total = st.cum[st.paths];
     const int nsplit = split ? __ldg(split) : 0;
     const bool on = split && nsplit <= scap;
     if ((int)blockIdx.x < scap) {
         if (!on || (int)blockIdx.x >= nsplit) return;
-        float *bufA = sm + 1;
+        float *bufA = sm + 4;                   // the split rows on 16-byte boundaries, Gs + 8 floats
         sgm_scanline<REC, true, WPC>(cost, lo, cnt, off, H, W, P1, P2, G, agg, status, __ldg(split + 1 + blockIdx.x),
-                                     mk, codes, amin, nnz_cap, bufA, bufA + (Gs + 2), meta, xm, wib);
+                                     mk, codes, amin, nnz_cap, bufA, bufA + (Gs + 8), meta, xm, wib,
+                                     bufA + 2 * (Gs + 8), Gs + 8);
         return;
     }
     const int gw = ((int)blockIdx.x - scap) * WPC + wib;
+    if constexpr (PAIR) {
+        if (__ldg(split + 1 + scap + total) <= pair_wide) {
+            if (2 * gw >= total) return;
+            const int q = 2 * gw + ((threadIdx.x >> 4) & 1);
+            const int rs = q < total ? __ldg(order + q) : 0;
+            const bool have = q < total && !(on && __ldg(split + 1 + scap + scan_base(st, rs & 15) + (rs >> 4)) >= min_wide);
+            sgm_pair(cost, lo, cnt, off, H, W, P1, P2, G, agg, status, rs, have, mk,
+                     sm + (size_t)wib * 3 * (Gs + 8) + 4, Gs + 8, ring + 128 * wib);
+            return;
+        }
+    }
     if (gw >= total) return;
     const int rs = __ldg(order + gw);            // longest scanlines first
-    if (on && __ldg(split + 1 + scap + st.cum[rs & 15] + (rs >> 4))) return;
+    if (on && __ldg(split + 1 + scap + st.cum[rs & 15] + (rs >> 4)) >= min_wide) return;
     float *bufA = sm + (size_t)wib * 2 * (Gs + 2) + 1;
     sgm_scanline<REC, false, 1>(cost, lo, cnt, off, H, W, P1, P2, G, agg, status, rs, mk, codes, amin, nnz_cap,
                                 bufA, bufA + (Gs + 2), meta, xm, wib);
 }
 
-// The scanlines to split: one warp per scanline counts the windows wider than 32 labels on it
-// (128 steps per round, their loads issued together) and marks it (mark[id] = 1 when listed, 0
-// otherwise, for every scanline); one that reaches min_wide is listed (split[0] zeroed before,
-// up to scap of them: the list's order does not matter, every scanline's values are its own).
-// Warp w0 of nwarps (every lane of the warp calls it).
-__device__ __forceinline__ void split_list(const int *__restrict__ cnt, int H, int W, const ScanTable &st,
-                                           int min_wide, int scap, int *__restrict__ split, int w0, int nwarps) {
-    const int lane = threadIdx.x & 31;
-    const int total = st.cum[st.paths];
-    int *mark = split + 1 + scap;
-    for (int id = w0; id < total; id += nwarps) {
-        // the direction: unrolled compares with the table (a run-time index would copy it to the stack)
-        int r = 0, base = 0;
-#pragma unroll
-        for (int q = 1; q < kMaxPaths; q++)
-            if (q < st.paths && id >= st.cum[q]) {
-                r = q;
-                base = st.cum[q];
-            }
-        const int s = id - base;
+// The scanlines to split: every pixel with a window wider than 32 labels counts on its scanline of each
+// direction (tab[1 + kSplitCap + id]); the one that reaches min_wide lists the scanline (tab[0] listed,
+// tab[1 .. kSplitCap] the list, up to kSplitCap of them: the list's order does not matter, every
+// scanline's values are its own).  Table zeroed before.  Such pixels are few where splitting pays, so
+// this costs the kernels that walk the windows anyway (mean cost, clearing the aggregate) no time; a
+// warp per scanline that counts them took 10 us for 8 directions of 512^2, 15 for 16 of 720 x 1280.
+// Called by a warp, lane i with pixel p0 + i, wide: its pixels with such windows; the lanes take
+// (pixel, direction) pairs, so that a few pixels wait for one round of atomics.
+__device__ __forceinline__ void count_wide(unsigned wide, int p0, int W, int H, const ScanTable &st, int min_wide,
+                                           int *tab) {
+    if (wide == 0u) return;
+    const int lane = threadIdx.x & 31, items = __popc(wide) * st.paths;
+    if (lane == 0) atomicAdd(tab + 1 + kSplitCap + st.cum[st.paths], __popc(wide));
+    if (__ldcg(tab) > kSplitCap) return;                   // too many listed: none is split
+    for (int i = lane; i < items; i += 32) {
+        const int k = st.paths == 8 ? i >> 3 : i >> 4, r = i - k * st.paths;
+        const int p = p0 + (int)__fns(wide, 0, k + 1);
+        const int y = p / W, x = p - y * W;
         int dx, dy;
         dir_of(r, dx, dy);
-        int x0, y0;
-        scan_start_d(dx, dy, s, H, W, x0, y0);
-        const int len = scan_steps(x0, y0, dx, dy, H, W);
-        const long long p0 = (long long)y0 * W + x0, dp = (long long)dy * W + dx;
-        int c = 0;
-        for (int k0 = 0; k0 < len; k0 += 128) {
-            int v[4];
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int k = k0 + 32 * u + lane;
-                v[u] = k < len ? __ldg(cnt + p0 + k * dp) : 0;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; u++) c += v[u] > 32;
-        }
-        c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-        if (lane == 0) {
-            int listed = 0;
-            if (c >= min_wide) {
-                const int pos = atomicAdd(split, 1);
-                if (pos < scap) {
-                    split[1 + pos] = (s << 4) | r;
-                    listed = 1;
-                }
-            }
-            mark[id] = listed;
+        const int base = scan_base(st, r);
+        const int q = scan_index_d(dx, dy, x, y, H, W);
+        if (atomicAdd(tab + 1 + kSplitCap + base + q, 1) == min_wide - 1) {
+            const int pos = atomicAdd(tab, 1);
+            if (pos < kSplitCap) tab[1 + pos] = (q << 4) | r;
         }
     }
 }
 
-__global__ void sgm_split_kernel(const int *__restrict__ cnt, int H, int W, ScanTable st, int min_wide, int scap,
-                                 int *__restrict__ split) {
-    split_list(cnt, H, W, st, min_wide, scap, split, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-               (gridDim.x * blockDim.x) >> 5);
+// The aggregate's rows to zero; with tab, the scanlines to split (count_wide).
+__global__ void __launch_bounds__(256) zero_agg_kernel(float *__restrict__ agg, const int *__restrict__ cnt,
+                                                       const long long *__restrict__ off, int N, int W, int H,
+                                                       ScanTable st, int min_wide, int *__restrict__ tab) {
+    const long long n = off[N], i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    if (tab)
+        for (long long p = i0; p - (threadIdx.x & 31) < N; p += stride)
+            count_wide(__ballot_sync(0xffffffffu, p < N && __ldg(cnt + p) > 32), (int)p - (threadIdx.x & 31), W, H, st,
+                       min_wide, tab);
+    zero_rows(agg, n, i0, stride);
 }
 
 // Per-block sums of the active costs and slot counts (rows are 16-byte aligned, read as float4;
@@ -516,29 +841,20 @@ __global__ void sgm_split_kernel(const int *__restrict__ cnt, int H, int W, Scan
 // order), so that one wide row does not hold its warp for a dependent load per 32 slots.  Each
 // lane adds its pixels in a fixed order, the block adds its warps in a fixed order, and the last
 // block to finish (ticket counter) adds the block partials in block order and writes the
-// penalties: the mean is deterministic.  The first nb blocks do this; blocks past them (split not
-// null) list the SGM scanlines to split (split_list, split[0] zeroed before), beside them.
+// penalties: the mean is deterministic.  The first nb blocks do this and, with tab, list the SGM
+// scanlines to split (count_wide); the blocks past them set the aggregate's rows to 0, beside sums
+// that wait for memory (9x9 x 512^2: 33 + 10 us as two kernels, 36 in one).
 __global__ void __launch_bounds__(256) cost_partial_kernel(const float *__restrict__ cost,
                                                            const int *__restrict__ cnt,
                                                            const long long *__restrict__ off, int N, int G,
                                                            double *__restrict__ partial, int nb, double p1f,
                                                            double p2f, float *__restrict__ pen,
                                                            unsigned *__restrict__ ticket, int *__restrict__ status,
-                                                           int H, int W, ScanTable st, int min_wide, int scap,
-                                                           int *__restrict__ split, int nsplit,
-                                                           float *__restrict__ agg) {
-    if ((int)blockIdx.x >= nb + nsplit) {
-        // the aggregate's rows to 0, beside the sums (which wait for memory)
-        const long long n4 = off[N] >> 2, stride = (long long)((int)gridDim.x - nb - nsplit) * blockDim.x;
-        float4 *z = reinterpret_cast<float4 *>(agg);
-        for (long long i = (long long)((int)blockIdx.x - nb - nsplit) * blockDim.x + threadIdx.x; i < n4; i += stride)
-            z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (long long i = 4 * n4 + threadIdx.x; i < off[N]; i += blockDim.x) agg[i] = 0.f;
-        return;
-    }
+                                                           int H, int W, ScanTable st, int min_wide,
+                                                           int *__restrict__ tab, float *__restrict__ agg) {
     if ((int)blockIdx.x >= nb) {
-        split_list(cnt, H, W, st, min_wide, scap, split, (((int)blockIdx.x - nb) * blockDim.x + threadIdx.x) >> 5,
-                   (nsplit * blockDim.x) >> 5);
+        zero_rows(agg, off[N], (long long)((int)blockIdx.x - nb) * blockDim.x + threadIdx.x,
+                  (long long)((int)gridDim.x - nb) * blockDim.x);
         return;
     }
     double s = 0.0, c = 0.0;
@@ -570,6 +886,7 @@ __global__ void __launch_bounds__(256) cost_partial_kernel(const float *__restri
         // a time; when most rows are wide (whole-range searches) each lane sums its own in 32-slot
         // chunks of 8 vector loads issued together
         unsigned wide = __ballot_sync(0xffffffffu, n > 32);
+        if (tab) count_wide(wide, base, W, H, st, min_wide, tab);
         if (__popc(wide) > 4) {
             for (int j0 = 32; j0 < n; j0 += 32) {
 #pragma unroll
@@ -663,20 +980,16 @@ __global__ void __launch_bounds__(256) cost_partial_kernel(const float *__restri
 cudaError_t launch_cost_partial_sums(cudaStream_t s, const float *cost, const int *cnt, const long long *off,
                                      int N, int G, double *partial, int nblocks, double p1f, double p2f,
                                      float *pen, unsigned *ticket, int *status, int H, int W, int paths,
-                                     int min_wide, int *split, float *agg) {
-    const ScanTable st = make_scan_table(H, W, paths);
-    int extra = 0;
-    if (split) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        extra = std::min((st.cum[paths] + 7) / 8, sms * 8);      // a warp per scanline
-    }
+                                     int min_wide, int *tab, float *agg) {
     // zeroing: a thread per 8 vectors of rows of about 32 slots, four CTAs per SM at most
-    const int zero = agg ? std::max(1, std::min(608, N / 256)) : 0;
-    cost_partial_kernel<<<nblocks + extra + zero, 256, 0, s>>>(cost, cnt, off, N, G, partial, nblocks, p1f, p2f, pen,
-                                                               ticket, status, H, W, st, min_wide, kSplitCap, split,
-                                                               extra, agg);
+    const int zero = std::max(1, std::min(608, N / 256));
+    cost_partial_kernel<<<nblocks + zero, 256, 0, s>>>(cost, cnt, off, N, G, partial, nblocks, p1f, p2f, pen, ticket,
+                                                       status, H, W, make_scan_table(H, W, paths), min_wide, tab, agg);
+    return cudaGetLastError();
+}
+cudaError_t launch_zero_agg(cudaStream_t s, float *agg, const int *cnt, const long long *off, int H, int W, int paths,
+                            int min_wide, int *tab) {
+    zero_agg_kernel<<<1216, 256, 0, s>>>(agg, cnt, off, H * W, W, H, make_scan_table(H, W, paths), min_wide, tab);
     return cudaGetLastError();
 }
 
@@ -690,32 +1003,29 @@ void build_scan_order(int H, int W, int paths, std::vector<int> &order) {
 }
 
 int sgm_split_ints(int H, int W, int paths) {
-    return 1 + kSplitCap + make_scan_table(H, W, paths).cum[paths];
-}
-
-cudaError_t launch_sgm_split(cudaStream_t s, const int *cnt, int H, int W, int paths, int min_wide, int *split) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const ScanTable st = make_scan_table(H, W, paths);
-    const int want = (st.cum[paths] + 7) / 8;                 // a warp per scanline
-    sgm_split_kernel<<<min(want, sms * 8), 256, 0, s>>>(cnt, H, W, st, min_wide, kSplitCap, split);
-    return cudaGetLastError();
+    return 1 + kSplitCap + make_scan_table(H, W, paths).cum[paths] + 1;
 }
 
 cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, const int *cnt,
                             const long long *off, int H, int W, int G, const float *pen, float *agg,
                             int *status, const int *order, int paths, unsigned char *codes, int *amin,
-                            size_t nnz_cap, int warps_per_cta, const int *split) {
+                            size_t nnz_cap, int warps_per_cta, int min_wide, const int *split, bool narrow) {
     const int wpc = warps_per_cta == 2 || warps_per_cta == 8 ? warps_per_cta : kSgmWarps;
     const ScanTable st = make_scan_table(H, W, paths);
     const int Gs = (G + 31) & ~31;
-    const size_t smem = (size_t)wpc * (2 * (Gs + 2) * sizeof(float) + 64 * sizeof(int2)) + (size_t)(4 * wpc + 4) * 4;
+    // two scanlines a warp: windows of at most 32 labels where the initial map holds, enough scanlines to keep
+    // the SMs busy, and rows that leave room for as many CTAs as the registers do
+    const size_t rest = (size_t)(4 * wpc + 4) * 4;
+    const size_t psmem = row_floats(wpc, Gs, split, true) * sizeof(float) + (size_t)wpc * 128 * sizeof(int2) + rest;
+    const bool pair = split && narrow && !codes && st.cum[paths] >= kPairFrom && psmem * 28 <= (size_t)wpc * 224 * 1024;
+    const size_t smem =
+        pair ? psmem : row_floats(wpc, Gs, split, false) * sizeof(float) + (size_t)wpc * 64 * sizeof(int2) + rest;
     const int scap = split ? kSplitCap : 0;
     const unsigned grid = (unsigned)(scap + (st.cum[paths] + wpc - 1) / wpc);
     // one instantiation per CTA size, each with its own register budget (launch bounds)
-    auto kern = codes ? (wpc == 2 ? fine_sgm_kernel<true, 2> : wpc == 8 ? fine_sgm_kernel<true, 8> : fine_sgm_kernel<true, 4>)
-                      : (wpc == 2 ? fine_sgm_kernel<false, 2> : wpc == 8 ? fine_sgm_kernel<false, 8> : fine_sgm_kernel<false, 4>);
+#define LFSGM_FINE(R, P) (wpc == 2 ? fine_sgm_kernel<R, 2, P> : wpc == 8 ? fine_sgm_kernel<R, 8, P> : fine_sgm_kernel<R, 4, P>)
+    auto kern = codes ? LFSGM_FINE(true, false) : pair ? LFSGM_FINE(false, true) : LFSGM_FINE(false, false);
+#undef LFSGM_FINE
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -724,7 +1034,7 @@ cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, co
     while ((1 << lp) < paths) lp++;
     const int mk = (lp << 23) | (1 << 22);       // (23 - qsh) << 23 with qsh = 23 - log2(paths)
     kern<<<grid, 32 * wpc, smem, s>>>(cost, lo, cnt, off, H, W, Gs, pen, G, st, agg, status, order, mk, codes,
-                                      amin, nnz_cap, split, scap);
+                                      amin, nnz_cap, split, scap, min_wide, H * W / 100);
     return cudaGetLastError();
 }
 

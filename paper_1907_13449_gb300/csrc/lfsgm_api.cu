@@ -61,7 +61,7 @@ struct lfsgm_ctx {
     // tuning knobs (lfsgm_set_tuning): label span of the row kernel's ranges, list-kernel CTAs per SM
     int row_kw = 36, list_ctas = 0, sgm_warps = 4;
     // scanlines that cross at least this many windows wider than 32 labels run split across a CTA's
-    // warps (lfsgm_set_sgm_split; 0: none)
+    // warps (lfsgm_set_sgm_split; 0: see split_from)
     int sgm_split = 0;
     std::vector<FineTap> h_fine;          // host copy of the shift table (row descriptors are rebuilt from it)
     // device tables
@@ -752,25 +752,33 @@ lfsgm_status lfsgm_cost_volume(lfsgm_handle h, const float *views, const int32_t
 }  // extern "C"
 
 namespace {
-// The aggregate's rows (and the first nz ints of the SGM's split table) to zero.
-__global__ void zero_csr_kernel(float *a, const long long *off, int N, int *z, int nz) {
-    const long long n = off[N];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        a[i] = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nz; i += gridDim.x * blockDim.x) z[i] = 0;
-}
-
-// Zero the aggregate, then (with the split knob on, and `list`) list the SGM scanlines to split.
-lfsgm_status sgm_prologue(lfsgm_ctx *h, float *agg, const int32_t *cnt, const long long *o, bool list) {
-    cudaStream_t s = h->stream;
+// Windows wider than 32 labels from which on a scanline runs split across a CTA (0: none does).  Where
+// the caller has set no threshold: 24, unless scanlines are short (a scanline of 256 steps with 24 such
+// windows takes about as long as one of 340 without) or every window is the whole range (then all are
+// alike).  Two scanlines of 9x9 x 512^2 cross 147 windows of 401 labels each and outlast all others:
+// 297 us without, 242 with the split (24, 48 and 96 alike, 215 with vectors of four labels; recording 382
+// and 313); the same time without such scanlines.  8 or 12 list more than the table holds.
+int split_from(const lfsgm_ctx *h) {
     const lfsgm_config &c = h->cfg;
-    const int nz = h->sgm_split > 0 ? 1 : 0;      // the split table's list count
-    LFSGM_TRY(run(h, "zero_agg", [&] {
-        zero_csr_kernel<<<1216, 256, 0, s>>>(agg, o, h->N, h->split, nz);
-        return cudaGetLastError();
-    }));
-    if (nz == 0 || !list) return LFSGM_OK;
-    return run(h, "sgm_split", [&] { return launch_sgm_split(s, cnt, c.H, c.W, c.paths, h->sgm_split, h->split); });
+    if (h->sgm_split > 0) return h->sgm_split;
+    return !c.boundless && std::max(c.H, c.W) >= 256 ? 24 : 0;
+}
+// The split table cleared for the launch that lists the scanlines.
+lfsgm_status clear_split(lfsgm_ctx *h) {
+    if (split_from(h) == 0) return LFSGM_OK;
+    const cudaError_t e =
+        cudaMemsetAsync(h->split, 0, (size_t)sgm_split_ints(h->cfg.H, h->cfg.W, h->cfg.paths) * 4, h->stream);
+    return e == cudaSuccess ? LFSGM_OK : cuda_fail(h, e, "memset");
+}
+int *split_table(lfsgm_ctx *h) { return split_from(h) > 0 ? h->split : nullptr; }
+
+// Explicit penalties: zero the aggregate and list the scanlines to split.
+lfsgm_status sgm_prologue(lfsgm_ctx *h, float *agg, const int32_t *cnt, const long long *o) {
+    const lfsgm_config &c = h->cfg;
+    LFSGM_TRY(clear_split(h));
+    return run(h, "zero_agg", [&] {
+        return launch_zero_agg(h->stream, agg, cnt, o, c.H, c.W, c.paths, split_from(h), split_table(h));
+    });
 }
 __global__ void set_pen_kernel(float *pen, float P1, float P2) {
     pen[0] = P1;
@@ -793,25 +801,24 @@ lfsgm_status lfsgm_sgm_aggregate(lfsgm_handle h, const float *cost, const int32_
     cudaStream_t s = h->stream;
     const long long *o = (const long long *)off;
     if (derived) {
-        // the penalty mean, whose launch also zeroes agg; with the split knob on, agg and the split list's
-        // count are zeroed first, and the launch lists the scanlines to split
-        if (h->sgm_split > 0) LFSGM_TRY(sgm_prologue(h, agg, cnt, o, false));
+        // the penalty mean, whose launch also zeroes agg and lists the scanlines to split
+        LFSGM_TRY(clear_split(h));
         LFSGM_TRY(run(h, "cost_partial_sums", [&] {
             return launch_cost_partial_sums(s, cost, cnt, o, h->N, c.fine_labels, h->partial, kPartialBlocks,
                                             c.p1_frac, c.p2_frac, h->fpen, h->ticket, h->status, c.H, c.W,
-                                            c.paths, h->sgm_split, h->sgm_split > 0 ? h->split : nullptr,
-                                            h->sgm_split > 0 ? nullptr : agg);
+                                            c.paths, split_from(h), split_table(h), agg);
         }));
     } else {
         LFSGM_TRY(run(h, "set_penalties", [&] {
             set_pen_kernel<<<1, 1, 0, s>>>(h->fpen, P1, P2);
             return cudaGetLastError();
         }));
-        LFSGM_TRY(sgm_prologue(h, agg, cnt, o, true));
+        LFSGM_TRY(sgm_prologue(h, agg, cnt, o));
     }
     LFSGM_TRY(run(h, "fine_sgm", [&] {
         return launch_fine_sgm(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, h->fpen, agg, h->status, h->d_order,
-                               c.paths, nullptr, nullptr, 0, h->sgm_warps, h->sgm_split > 0 ? h->split : nullptr);
+                               c.paths, nullptr, nullptr, 0, h->sgm_warps, split_from(h), split_table(h),
+                               2 * std::max(c.fine_radius, c.fine_radius_far) < 32);
     }));
     return LFSGM_OK;
 }
@@ -864,11 +871,11 @@ static lfsgm_status aggregate_recording(lfsgm_handle h, const float *cost, const
         set_pen_kernel<<<1, 1, 0, s>>>(h->fpen, P1, P2);
         return cudaGetLastError();
     }));
-    LFSGM_TRY(sgm_prologue(h, agg, cnt, o, true));
+    LFSGM_TRY(sgm_prologue(h, agg, cnt, o));
     return run(h, "fine_sgm_record", [&] {
         return launch_fine_sgm(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, h->fpen, agg, h->status, h->d_order,
                                c.paths, h->b_codes, h->b_amin, (size_t)cap, h->sgm_warps,
-                               h->sgm_split > 0 ? h->split : nullptr);
+                               split_from(h), split_table(h));
     });
 }
 
@@ -1103,34 +1110,29 @@ lfsgm_status tune_handle(lfsgm_handle h, const float *views, int32_t *lo, int32_
     if (st == LFSGM_OK) st = lfsgm_set_tuning(h, best_kw, best_lc);
     // the SGM's warps (scanlines) per CTA, on the cost volume of the chosen knobs (derived penalties)
     if (st == LFSGM_OK) st = cost_volume_impl(h, views, lo, cnt, off, cost, !h->cfg.boundless);
-    // and whether scanlines that cross many wide windows run split across a CTA (off or threshold 24)
-    int best_w = 4, best_sp = 0;
+    int best_w = 4;
     float best_sgm = 1e30f;
-    for (int w : {4, 8, 2})
-        for (int sp : {0, 24}) {
-            if (st != LFSGM_OK) break;
-            st = lfsgm_set_sgm_warps(h, w);
-            if (st == LFSGM_OK) st = lfsgm_set_sgm_split(h, sp);
-            float best = 1e30f;
-            for (int r = 0; r < 3 && st == LFSGM_OK; r++) {
-                cudaEventRecord(e0, h->stream);
-                st = lfsgm_sgm_aggregate(h, cost, lo, cnt, off, -1.f, -1.f, agg);
-                cudaEventRecord(e1, h->stream);
-                cudaEventSynchronize(e1);
-                float t = 0.f;
-                cudaEventElapsedTime(&t, e0, e1);
-                if (r > 0) best = std::min(best, t);
-            }
-            if (st == LFSGM_OK && best < best_sgm) {
-                best_sgm = best;
-                best_w = w;
-                best_sp = sp;
-            }
+    for (int w : {4, 8, 2}) {
+        if (st != LFSGM_OK) break;
+        st = lfsgm_set_sgm_warps(h, w);
+        float best = 1e30f;
+        for (int r = 0; r < 3 && st == LFSGM_OK; r++) {
+            cudaEventRecord(e0, h->stream);
+            st = lfsgm_sgm_aggregate(h, cost, lo, cnt, off, -1.f, -1.f, agg);
+            cudaEventRecord(e1, h->stream);
+            cudaEventSynchronize(e1);
+            float t = 0.f;
+            cudaEventElapsedTime(&t, e0, e1);
+            if (r > 0) best = std::min(best, t);
         }
+        if (st == LFSGM_OK && best < best_sgm) {
+            best_sgm = best;
+            best_w = w;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st == LFSGM_OK) st = lfsgm_set_sgm_warps(h, best_w);
-    if (st == LFSGM_OK) st = lfsgm_set_sgm_split(h, best_sp);
     kw_out = best_kw;
     lc_out = best_lc;
     return st;
