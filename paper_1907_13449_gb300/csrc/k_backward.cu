@@ -3,14 +3,17 @@
 // Loss gradients arrive as grad_disp = dLoss/d dhat(p) for the soft-argmin disparity
 // dhat = sum_g softmax(-C_s/tau)_g d_g.  Three kernels:
 //  * softargmin_backward: dLoss/dC_s(p,g) = grad_disp(p) (-1/tau) w_g (d_g - dhat).
-//  * sgm_backward: one warp per (direction, scanline).  The path is recomputed forward, recording
-//    for every cell the winning branch of the normalised recurrence (P2 first, then same, g-1,
-//    g+1, taken with strict comparisons in that order) and for every pixel the slot of its
-//    minimum; the reverse sweep carries lambda = dLoss/dL_r along the path: it adds lambda into
-//    dLoss/dC, gathers the predecessor's incoming adjoint from the three slots whose branch points
-//    at it, routes (P2-branch lambdas - all lambdas) to the predecessor's minimum (the -m term),
-//    and sums the branch lambdas into dLoss/dP1, dLoss/dP2.  Path costs are recomputed per
-//    direction instead of being stored for all 8.
+//  * sgm_backward: one warp per (direction, scanline), on what the recording forward wrote: for every
+//    cell the winning branch of the normalised recurrence (P2 first, then same, g-1, g+1, taken with
+//    strict comparisons in that order) and for every pixel the slot of its minimum.  The reverse
+//    sweep carries lambda = dLoss/dL_r along the path: it adds lambda into dLoss/dC, gathers the
+//    predecessor's incoming adjoint from the three slots whose branch points at it, routes
+//    (P2-branch lambdas - all lambdas) to the predecessor's minimum (the -m term), and sums the
+//    branch lambdas into dLoss/dP1, dLoss/dP2.  What bounds it: the scanlines that cross the most
+//    wide windows (9x9 x 512^2: 147 of 401 labels, the others were done at 0.6 of the time):
+//    840 us with a label a lane, the predecessor's argmin and the codes loaded where they are used; 555
+//    with vectors of four labels, and with routed values instead of values and codes in the narrow
+//    step's shuffles.
 //  * views_backward: one warp per (pixel, 32-label chunk); dC/dI_ref = w_l2 sum sign(I_ref - B),
 //    dC/dI_v(tap) = -w_l2 sign(.) w_tap (taps clamped as in the forward); lanes of one bilinear
 //    cell are summed by a segmented shuffle and added to the view with four atomics per cell.
@@ -75,12 +78,10 @@ __global__ void __launch_bounds__(256) softargmin_backward_kernel(const float *_
 
 // Branch codes: 0 same label, 1 label-1 (+P1), 2 label+1 (+P1), 3 m+P2, 4 path start.
 __global__ void __launch_bounds__(32 * kBwdWarps) sgm_backward_kernel(
-    const float *__restrict__ cost, const int *__restrict__ lo, const int *__restrict__ cnt,
-    const long long *__restrict__ off, int H, int W, int G, int Gs, float P1, float P2, ScanTable st,
-    const float *__restrict__ gCs, unsigned char *__restrict__ codes, int *__restrict__ amin, size_t nnz_cap,
-    float *__restrict__ gcost, float *__restrict__ gP, int *__restrict__ status,
-    const int *__restrict__ order, int recompute) {
-    extern __shared__ float sm[];
+    const int *__restrict__ lo, const int *__restrict__ cnt, const long long *__restrict__ off, int H, int W, int G, int Gs,
+    ScanTable st, const float *__restrict__ gCs, const unsigned char *__restrict__ codes, const int *__restrict__ amin,
+    size_t nnz_cap, float *__restrict__ gcost, float *__restrict__ gP, const int *__restrict__ order) {
+    extern __shared__ __align__(16) float sm[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int gw = blockIdx.x * kBwdWarps + wib;
     if (gw >= st.cum[st.paths]) return;
@@ -90,162 +91,49 @@ __global__ void __launch_bounds__(32 * kBwdWarps) sgm_backward_kernel(
     int x0, y0;
     scan_start(r, s, H, W, x0, y0);
     const int len = scan_steps(x0, y0, dx, dy, H, W);
-    unsigned char *code = codes + (size_t)r * nnz_cap;
-    int *am = amin + (size_t)r * H * W;
-    float *bufA = sm + (size_t)wib * 4 * Gs;   // forward: predecessor's L;  reverse: incoming adjoint of p
-    float *bufB = bufA + Gs;                   // forward: this pixel's L;    reverse: incoming adjoint of q
-    float *lam = bufB + Gs;                    // reverse: lambda of p by slot
-    unsigned char *cds = (unsigned char *)(lam + Gs);
-    const float INF = __int_as_float(0x7f800000);
+    const unsigned char *code = codes + (size_t)r * nnz_cap;
+    const int *am = amin + (size_t)r * H * W;
+    float *bufA = sm + (size_t)wib * 4 * Gs;   // incoming adjoint of p by slot
+    float *bufB = bufA + Gs;                   // incoming adjoint of q
+    float *lam = bufB + Gs;                    // lambda of p
+    unsigned char *cds = (unsigned char *)(lam + Gs);   // and the branch codes
 
     // window metadata of 32 steps per lane: (lo | cnt << 16), 0 for an invalid window, and the
     // row offset in units of 4 slots; the next block is fetched one block ahead
     const long long p0 = (long long)y0 * W + x0, dpix = (long long)dy * W + dx;
-    auto fetch = [&](int kb, int &mw, int &mo, int *st_) {
+    auto fetch = [&](int kb, int &mw, int &mo) {
         const int k = kb + lane;
         mw = 0;
         mo = 0;
         if (k >= 0 && k < len) {
             const long long p = p0 + (long long)k * dpix;
             const int l_ = __ldg(lo + p), n_ = __ldg(cnt + p);
-            const long long o_ = __ldg(off + p);
-            if (window_ok(l_, n_, G, __ldg(off + p + 1) - o_, st_) && (o_ & 3) == 0 && (o_ >> 2) < 0x7fffffff) {
+            const long long o_ = __ldg(off + p), e_ = __ldg(off + p + 1);
+            if (window_ok(l_, n_, G, e_ - o_, nullptr) && ((o_ | e_) & 3) == 0 && (o_ >> 2) < 0x7fffffff) {
                 mw = l_ | (n_ << 16);
                 mo = (int)(o_ >> 2);
             }
         }
     };
 
-    // forward recompute: branch codes and argmin slots (recompute = 1; the library passes 0, as the
-    // forward SGM's recording form writes them.  The path is kept: without it the compiler
-    // allocates the reverse sweep differently and it ran 4 % slower, 0.708 vs 0.681 ms.)  Narrow
-    // steps (this window and the predecessor's at most 32 labels) keep the predecessor row in
-    // registers, one slot per lane, and take its neighbours by shuffles; wider ones use the rows in
-    // shared memory.
-    int plo = 0, pn = 0;
-    float m = 0.f;
-    bool first = true;
-    float prev = INF;                          // predecessor row by slot (narrow form)
-    bool in_smem = false;                      // the predecessor row is in bufA (general form)
-    int cw, co, nw = 0, no = 0;
-    fetch(0, cw, co, status);
-    if (len > 32) fetch(32, nw, no, status);
-    for (int k = 0; k < (recompute ? len : 0); k++) {
-        const int kk = k & 31;
-        if (kk == 0 && k > 0) {
-            cw = nw;
-            co = no;
-            if (k + 32 < len) fetch(k + 32, nw, no, status);
-        }
-        const int win = __shfl_sync(0xffffffffu, cw, kk), ofs = __shfl_sync(0xffffffffu, co, kk);
-        const int p = (int)(p0 + (long long)k * dpix);
-        const int l = win & 0xffff, n = win >> 16;
-        const long long o = 4ll * ofs;
-        if (n == 0) {
-            first = true;
-            continue;
-        }
-        if (n <= 32 && (first || pn <= 32)) {
-            if (!first && in_smem) prev = lane < pn ? bufA[lane] : INF;
-            const float c = lane < n ? __ldg(cost + o + lane) : 0.f;
-            float Lv = c;
-            unsigned cd = 4;
-            if (!first) {
-                // the same candidates in the same order as the general form: P2, same, g-1, g+1
-                const int i = lane + (l - plo);
-                const float v0 = __shfl_sync(0xffffffffu, prev, i & 31);
-                const float vm = __shfl_sync(0xffffffffu, prev, (i - 1) & 31);
-                const float vp = __shfl_sync(0xffffffffu, prev, (i + 1) & 31);
-                float t = m + P2;
-                cd = 3;
-                if ((unsigned)i < (unsigned)pn && v0 < t) { t = v0; cd = 0; }
-                if ((unsigned)(i - 1) < (unsigned)pn && vm + P1 < t) { t = vm + P1; cd = 1; }
-                if ((unsigned)(i + 1) < (unsigned)pn && vp + P1 < t) { t = vp + P1; cd = 2; }
-                Lv = c + (t - m);
-            }
-            if (lane < n) code[o + lane] = (unsigned char)cd;
-            const float bv = lane < n ? Lv : INF;
-            float mv;
-            asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(mv) : "f"(bv));
-            const int slot = __reduce_min_sync(0xffffffffu, bv == mv ? (unsigned)lane : 0x7fffffffu);
-            if (lane == 0) am[p] = slot;
-            m = mv;
-            prev = bv;
-            in_smem = false;
-            plo = l;
-            pn = n;
-            first = false;
-            continue;
-        }
-        if (!first && !in_smem) {
-            if (lane < pn) bufA[lane] = prev;
-            __syncwarp();
-        }
-        float bv = INF;
-        int bj = 0x7fffffff;
-        // eight 32-label chunks per round: their cost loads are in flight together
-        for (int j0 = lane; j0 < n; j0 += 256) {
-        float cv[8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) cv[u] = j0 + 32 * u < n ? __ldg(cost + o + j0 + 32 * u) : 0.f;
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int j = j0 + 32 * u;
-            if (j >= n) break;
-            const float c = cv[u];
-            float Lv;
-            unsigned char cd = 4;
-            if (first) {
-                Lv = c;
-            } else {
-                const int i = l + j - plo;
-                float t = m + P2;
-                cd = 3;
-                if ((unsigned)i < (unsigned)pn && bufA[i] < t) { t = bufA[i]; cd = 0; }
-                if ((unsigned)(i - 1) < (unsigned)pn && bufA[i - 1] + P1 < t) { t = bufA[i - 1] + P1; cd = 1; }
-                if ((unsigned)(i + 1) < (unsigned)pn && bufA[i + 1] + P1 < t) { t = bufA[i + 1] + P1; cd = 2; }
-                Lv = c + (t - m);
-            }
-            bufB[j] = Lv;
-            code[o + j] = cd;
-            if (Lv < bv) { bv = Lv; bj = j; }
-        }
-        }
-        // minimum and its lowest slot
-        float mv;
-        asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(mv) : "f"(bv));
-        const int cand = (bv == mv) ? bj : 0x7fffffff;
-        const int slot = __reduce_min_sync(0xffffffffu, (unsigned)cand);
-        if (lane == 0) am[p] = slot;
-        m = mv;
-        __syncwarp();
-        float *tmp = bufA;
-        bufA = bufB;
-        bufB = tmp;
-        in_smem = true;
-        plo = l;
-        pn = n;
-        first = false;
-    }
-    __syncwarp();
-
+    int cw, co, nw = 0, no = 0;                // a block's and the next (lower) block's metadata
     // reverse sweep (blocks of metadata in descending order; step k-1 is in this block or the one below)
     float gp1 = 0.f, gp2 = 0.f;
     bool have_inc = false;       // the current pixel has an incoming adjoint (from its successor)
     bool inc_smem = false;       // ... held in bufA by slot (general form), else in inc, one slot per lane
     float inc = 0.f;
-    // the argmin slot of each step of a block, fetched with its metadata (written above by this warp)
+    // the argmin slot of each step of a block, fetched with its metadata
     auto fetch_am = [&](int kb) {
         const int kq = kb + lane;
-        return (kq >= 0 && kq < len) ? am[(int)(p0 + (long long)kq * dpix)] : 0;
+        return (kq >= 0 && kq < len) ? __ldg(am + (int)(p0 + (long long)kq * dpix)) : 0;
     };
     int ca = 0, na = 0;
     {
         const int kb0 = (len - 1) & ~31;
-        fetch(kb0, cw, co, nullptr);
+        fetch(kb0, cw, co);
         ca = fetch_am(kb0);
         if (kb0 >= 32) {
-            fetch(kb0 - 32, nw, no, nullptr);
+            fetch(kb0 - 32, nw, no);
             na = fetch_am(kb0 - 32);
         }
     }
@@ -261,7 +149,7 @@ __global__ void __launch_bounds__(32 * kBwdWarps) sgm_backward_kernel(
             co = no;
             ca = na;
             if (kb >= 32) {
-                fetch(kb - 32, nw, no, nullptr);
+                fetch(kb - 32, nw, no);
                 na = fetch_am(kb - 32);
             }
         }
@@ -313,14 +201,14 @@ __global__ void __launch_bounds__(32 * kBwdWarps) sgm_backward_kernel(
             if (q >= 0) {
                 const int qa = __shfl_sync(0xffffffffu, kk > 0 ? ca : na, (kk + 31) & 31);
                 const int j0 = lane + (ql - l), j1 = j0 + 1, j2 = j0 - 1;
-                const float l0 = __shfl_sync(0xffffffffu, lv, j0 & 31), l1 = __shfl_sync(0xffffffffu, lv, j1 & 31);
-                const float l2 = __shfl_sync(0xffffffffu, lv, j2 & 31);
-                const unsigned c0 = __shfl_sync(0xffffffffu, cd, j0 & 31), c1 = __shfl_sync(0xffffffffu, cd, j1 & 31);
-                const unsigned c2 = __shfl_sync(0xffffffffu, cd, j2 & 31);
+                // lv (0 from slot n on) goes to the label, the one below or the one above that its code names
+                const float l0 = __shfl_sync(0xffffffffu, cd == 0 ? lv : 0.f, j0 & 31);
+                const float l1 = __shfl_sync(0xffffffffu, cd == 1 ? lv : 0.f, j1 & 31);
+                const float l2 = __shfl_sync(0xffffffffu, cd == 2 ? lv : 0.f, j2 & 31);
                 float v = 0.f;
-                if ((unsigned)j0 < (unsigned)n && c0 == 0) v += l0;
-                if ((unsigned)j1 < (unsigned)n && c1 == 1) v += l1;
-                if ((unsigned)j2 < (unsigned)n && c2 == 2) v += l2;
+                if ((unsigned)j0 < 32u) v += l0;
+                if ((unsigned)j1 < 32u) v += l1;
+                if ((unsigned)j2 < 32u) v += l2;
                 if (lane == qa) v += dm;
                 inc = lane < qn ? v : 0.f;
                 inc_smem = false;
@@ -334,47 +222,71 @@ __global__ void __launch_bounds__(32 * kBwdWarps) sgm_backward_kernel(
             if (lane < n) bufA[lane] = inc;
             __syncwarp();
         }
+        // four consecutive labels a lane, four such vectors of both inputs in flight together
         float dm = 0.f;
-        for (int j0 = lane; j0 < n; j0 += 256) {
-        float gv[8];
-        unsigned char cv[8];
+        for (int jr = 4 * lane; jr < n; jr += 512) {
+            float4 g4[4];
+            unsigned c4[4];
 #pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const bool in = j0 + 32 * u < n;
-            gv[u] = in ? __ldg(gCs + o + j0 + 32 * u) : 0.f;
-            cv[u] = in ? code[o + j0 + 32 * u] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int j = j0 + 32 * u;
-            if (j >= n) break;
-            const float lv = gv[u] + (have_inc ? bufA[j] : 0.f);
-            atomicAdd(gcost + o + j, lv);
-            const unsigned char cd = cv[u];
-            lam[j] = lv;
-            cds[j] = cd;
-            if (cd == 1 || cd == 2) gp1 += lv;
-            if (cd == 3) {
-                gp2 += lv;
-                dm += lv;
+            for (int u = 0; u < 4; u++) {
+                const bool in = jr + 128 * u < n;
+                g4[u] = in ? __ldg(reinterpret_cast<const float4 *>(gCs + o + jr + 128 * u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                c4[u] = in ? __ldg(reinterpret_cast<const unsigned *>(code + o + jr + 128 * u)) : 0u;
             }
-            dm -= lv;
-        }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int j = jr + 128 * u;
+                if (j >= n) break;
+                const float4 i4 = have_inc ? *reinterpret_cast<const float4 *>(bufA + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float lv[4] = {g4[u].x + i4.x, j + 1 < n ? g4[u].y + i4.y : 0.f, j + 2 < n ? g4[u].z + i4.z : 0.f,
+                                     j + 3 < n ? g4[u].w + i4.w : 0.f};
+                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
+                             ::"l"(gcost + o + j), "f"(lv[0]), "f"(lv[1]), "f"(lv[2]), "f"(lv[3]) : "memory");
+                *reinterpret_cast<float4 *>(lam + j) = make_float4(lv[0], lv[1], lv[2], lv[3]);
+                *reinterpret_cast<unsigned *>(cds + j) = c4[u];
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    const unsigned cd = c4[u] >> (8 * e) & 255u;
+                    if (cd == 1 || cd == 2) gp1 += lv[e];
+                    if (cd == 3)
+                        gp2 += lv[e];
+                    else
+                        dm -= lv[e];
+                }
+            }
         }
         dm = warp_sum(dm);
         __syncwarp();
         if (q >= 0) {
             // gather q's incoming adjoint: label h receives from p's labels h (same), h+1 (-1 branch), h-1 (+1 branch)
-            const int qa = am[q];
-            for (int i = lane; i < qn; i += 32) {
-                const int h = ql + i;
-                float v = 0.f;
-                const int j0 = h - l, j1 = h + 1 - l, j2 = h - 1 - l;
-                if ((unsigned)j0 < (unsigned)n && cds[j0] == 0) v += lam[j0];
-                if ((unsigned)j1 < (unsigned)n && cds[j1] == 1) v += lam[j1];
-                if ((unsigned)j2 < (unsigned)n && cds[j2] == 2) v += lam[j2];
-                if (i == qa) v += dm;
-                bufB[i] = v;
+            const int qa = __shfl_sync(0xffffffffu, kk > 0 ? ca : na, (kk + 31) & 31);
+            if (ql == l && qn == n) {
+                for (int i = 4 * lane; i < n; i += 128) {
+                    const float4 f = *reinterpret_cast<const float4 *>(lam + i);
+                    const unsigned c = *reinterpret_cast<const unsigned *>(cds + i);
+                    // labels i - 1 .. i + 4; lam is 0 in the padding slots
+                    const float x[6] = {i > 0 ? lam[i - 1] : 0.f, f.x, f.y, f.z, f.w, i + 4 < n ? lam[i + 4] : 0.f};
+                    const unsigned d[6] = {i > 0 ? cds[i - 1] : 4u, c & 255u, c >> 8 & 255u, c >> 16 & 255u, c >> 24,
+                                           i + 4 < n ? cds[i + 4] : 4u};
+                    float v[4];
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        v[e] = (d[e + 1] == 0 ? x[e + 1] : 0.f) + (d[e + 2] == 1 ? x[e + 2] : 0.f) +
+                               (d[e] == 2 ? x[e] : 0.f);
+                        if (i + e == qa) v[e] += dm;
+                    }
+                    *reinterpret_cast<float4 *>(bufB + i) = make_float4(v[0], v[1], v[2], v[3]);
+                }
+            } else {
+                for (int i = lane; i < qn; i += 32) {
+                    float v = 0.f;
+                    const int j0 = ql + i - l, j1 = j0 + 1, j2 = j0 - 1;
+                    if ((unsigned)j0 < (unsigned)n && cds[j0] == 0) v += lam[j0];
+                    if ((unsigned)j1 < (unsigned)n && cds[j1] == 1) v += lam[j1];
+                    if ((unsigned)j2 < (unsigned)n && cds[j2] == 2) v += lam[j2];
+                    if (i == qa) v += dm;
+                    bufB[i] = v;
+                }
             }
             __syncwarp();
             float *tmp = bufA;
@@ -883,10 +795,9 @@ cudaError_t launch_softargmin_backward(cudaStream_t s, const float *agg, const i
     return cudaGetLastError();
 }
 
-cudaError_t launch_sgm_backward(cudaStream_t s, const float *cost, const int *lo, const int *cnt, const long long *off,
-                                int H, int W, int G, float P1, float P2, const float *gCs, unsigned char *codes,
-                                int *amin, size_t nnz_cap, float *gcost, float *gP, int *status, const int *order, int paths,
-                                bool recompute) {
+cudaError_t launch_sgm_backward(cudaStream_t s, const int *lo, const int *cnt, const long long *off, int H, int W, int G,
+                                const float *gCs, const unsigned char *codes, const int *amin, size_t nnz_cap,
+                                float *gcost, float *gP, const int *order, int paths) {
     const ScanTable st = make_scan_table(H, W, paths);
     const int Gs = (G + 31) & ~31;
     const size_t smem = (size_t)kBwdWarps * 4 * Gs * sizeof(float);   // bufA, bufB, lambda, codes per warp
@@ -896,8 +807,8 @@ cudaError_t launch_sgm_backward(cudaStream_t s, const float *cost, const int *lo
                                                    (int)smem);
         if (e != cudaSuccess) return e;
     }
-    sgm_backward_kernel<<<grid, 32 * kBwdWarps, smem, s>>>(cost, lo, cnt, off, H, W, G, Gs, P1, P2, st, gCs, codes,
-                                                           amin, nnz_cap, gcost, gP, status, order, recompute ? 1 : 0);
+    sgm_backward_kernel<<<grid, 32 * kBwdWarps, smem, s>>>(lo, cnt, off, H, W, G, Gs, st, gCs, codes, amin, nnz_cap, gcost,
+                                                           gP, order);
     return cudaGetLastError();
 }
 

@@ -899,9 +899,8 @@ static lfsgm_status backward_from_record(lfsgm_handle h, const float *views, con
     if (e == cudaSuccess && grad_views) e = cudaMemsetAsync(grad_views, 0, (size_t)h->nviews * h->C * N * 4, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "memset");
     LFSGM_TRY(run(h, "sgm_backward", [&] {
-        return launch_sgm_backward(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, P1, P2, h->b_gcs, h->b_codes,
-                                   h->b_amin, (size_t)cap, grad_cost, h->b_gp, h->status, h->d_order, c.paths,
-                                   false);
+        return launch_sgm_backward(s, lo, cnt, o, c.H, c.W, c.fine_labels, h->b_gcs, h->b_codes, h->b_amin,
+                                   (size_t)cap, grad_cost, h->b_gp, h->d_order, c.paths);
     }));
     if (grad_views) {
         // the (pixel, 32-label chunk) items of windows wider than 32 labels; narrower ones by rows,

@@ -54,10 +54,9 @@ def test_default_split_gives_the_same_bits_as_none(gpu_lib, H, W, rows, cols, pe
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
 
 
-def _case(H, W, paths, kind):
+def _case(H, W, paths, kind, G=97):
     """Windows that stand still or step by a label, or that jump, of 1 to 32 labels; 'jumps' and 'rows' with
     wider ones (0.6 % of the pixels; two whole rows)."""
-    G = 97
     p = lfsynth.LFParams(U=3, V=3, H=H, W=W, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=9, fine_labels=G,
                          fine_radius=8, w_l2=1.0, w_census=1.0 / 24, subpixel=2, softmin_tau=0.1, paths=paths)
     rng = np.random.default_rng(H * W + paths)
@@ -90,12 +89,13 @@ def test_two_scanlines_a_warp_match_the_oracle(gpu_lib, H, W, paths, kind):
     assert err < RTOL, err
 
 
-# The branches that split scanlines record: the adjoint against the oracle's.  The bar is that of the other
+# The branches that split scanlines record, and the adjoint's wide steps (four labels a lane, 512 a round;
+# 97, 98, 100 and 601 labels): the adjoint against the oracle's.  The bar is that of the other
 # adjoint tests, for all but 1e-4 of the elements (decisions that FP32 rounding makes at a kink, as on the
 # bench band).
-@pytest.mark.parametrize("H,W", [(20, 260), (260, 21)])
-def test_split_scanlines_record_the_adjoints_branches(gpu_lib, H, W):
-    p, views, lo, cnt, gd = _case(H, W, 8, "rows")
+@pytest.mark.parametrize("H,W,G", [(20, 260, 97), (260, 21, 98), (12, 60, 100), (6, 40, 601)])
+def test_split_scanlines_record_the_adjoints_branches(gpu_lib, H, W, G):
+    p, views, lo, cnt, gd = _case(H, W, 8, "rows", G)
     cfg = oracle.make_cfg(p)
     off_o, cost_o = oracle.cost_volume(cfg, views, lo, cnt)
     P1, P2 = _penalties(cost_o)
