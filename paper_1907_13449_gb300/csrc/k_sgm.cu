@@ -392,64 +392,24 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                                         REC ? code + o : nullptr, lmin, lslot, bufB);
                     }
                 }
-                // sixteen of this warp's 32-label chunks per round: their cost loads are in flight
-                // together, and every chunk reads the predecessor row before any chunk stores its own
-                // (the compiler cannot tell bufA from bufB, so a store between them would order the
-                // chunks one after another)
-                constexpr int CS = 32;                 // slot stride between the chunks
-                for (int j0 = lane; !SPLIT && j0 < n; j0 += 16 * CS) {
-                    float cc[16];
+                // one warp: four vectors of four labels a lane per round, their cost loads in flight together
+                // (512^2 pixels, windows of 401 labels at 10 % and 30 % of them: 282 and 503 us, with a label a lane
+                // 303 and 565)
+                if constexpr (!SPLIT) {
+                    const bool same = l == plo && n == pn;
+                    const unsigned top = (unsigned)pn + 1u;
+                    for (int jr = 4 * lane; jr < n; jr += 512) {
+                        float4 c4[4];
 #pragma unroll
-                    for (int u = 0; u < 16; u++) cc[u] = j0 + CS * u < n ? __ldg(cost + o + j0 + CS * u) : 0.f;
-                    if (pn != 0) {
-                        // predecessor slot s read at row[s + 1] with s + 1 clamped (unsigned) to
-                        // pn + 1: any slot outside [0, pn) lands on a sentinel (+inf), so an absent
-                        // label drops out of the minimum (labels j >= n read in-bounds slots too)
-                        const unsigned top = (unsigned)pn + 1u;
-                        const float *row = bufA - 1;
-                        auto step = [&](int u, float v0, float vm, float vp) {
-                            const float t = fminf(fminf(m + P2, v0), fminf(vm, vp) + P1);
-                            if (REC)
-                                code[o + j0 + CS * u] = t == m + P2 ? 3 : (t == v0 ? 0 : (t == vm + P1 ? 1 : 2));
-                            const float Ln = cc[u] + (t - m);
-                            // the cell's cost cc[u] bounds its path costs (the global atomic does
-                            // not order the shared-memory reads of the other chunks)
-                            atomicAdd(agg + o + j0 + CS * u, det_addend(Ln, cc[u] + P2, mk));
-                            cc[u] = Ln;
-                        };
-                        if (l == plo && n == pn) {
-                            // the same window as the predecessor (a run of whole-range windows):
-                            // slot j's neighbours are slots j - 1 and j + 1, and the sentinels at
-                            // slots -1 and pn stand in for the absent ones
-                            const float *q = bufA + j0;
+                        for (int u = 0; u < 4; u++)
+                            c4[u] = jr + 128 * u < n ? __ldg(reinterpret_cast<const float4 *>(cost + o + jr + 128 * u))
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                            for (int u = 0; u < 16; u++) {
-                                if (j0 + CS * u >= n) break;
-                                step(u, q[CS * u], q[CS * u - 1], q[CS * u + 1]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int u = 0; u < 16; u++) {
-                                if (j0 + CS * u >= n) break;
-                                const unsigned k1 = (unsigned)(l + j0 + CS * u - plo + 1);
-                                step(u, row[min(k1, top)], row[min(k1 - 1u, top)], row[min(k1 + 1u, top)]);
-                            }
+                        for (int u = 0; u < 4; u++) {
+                            if (jr + 128 * u >= n) break;
+                            wide_cells<REC>(c4[u], jr + 128 * u, n, l, plo, pn, same, top, bufA, m, P1, P2, mk, agg + o,
+                                            REC ? code + o : nullptr, lmin, lslot, bufB);
                         }
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 16; u++) {
-                            if (j0 + CS * u >= n) break;
-                            atomicAdd(agg + o + j0 + CS * u, det_addend(cc[u], cc[u] + P2, mk));
-                            if (REC) code[o + j0 + CS * u] = 4;
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 16; u++) {
-                        const int j = j0 + CS * u;
-                        if (j >= n) break;
-                        bufB[j] = cc[u];
-                        if (REC && cc[u] < lmin) lslot = j;      // a lane's slots ascend: its first minimum
-                        lmin = fminf(lmin, cc[u]);
                     }
                 }
                 if (SPLIT) {
@@ -720,7 +680,7 @@ __device__ __forceinline__ void sgm_pair(const float *__restrict__ cost, const i
 // listed ones.  split: [0] scanlines listed, [1 .. scap] the list (rs), then the wide windows of each
 // scanline and, last, of the image (count_wide); more than scap listed: none is split.  PAIR: where the
 // image has at most pair_wide (1 %) wide windows, a warp takes two scanlines (sgm_pair), and the CTAs past
-// them have nothing to do: 512^2 pixels without wide windows 174 -> 143 us, 4x4 x 720 x 1280 with 16
+// them have nothing to do: 512^2 pixels without wide windows 174 -> 141 us, 4x4 x 720 x 1280 with 16
 // directions and 0.6 % of them 1163 -> 800 us, but with 2 % of them 212 -> 221 us and with 10 % 321 -> 425 us,
 // since both scanlines wait for the wide steps of either.
 // Resident CTAs per SM that the register budget must allow: what the one-warp path reaches on its
@@ -730,10 +690,10 @@ __host__ __device__ constexpr int sgm_min_ctas(bool rec, int wpc) {
     return rec ? (wpc == 2 ? 10 : wpc == 4 ? 5 : 2) : (wpc == 2 ? 14 : wpc == 4 ? 7 : 3);
 }
 
-// Floats of the rows of fine_sgm_kernel's CTA: two per warp (PAIR: three, with room for alignment), or what a
+// Floats of the rows of fine_sgm_kernel's CTA: two per warp (PAIR: three), slot 0 on 16-byte boundaries, or what a
 // split scanline takes (sgm_scanline).
 __host__ __device__ constexpr int row_floats(int wpc, int Gs, bool split, bool pair) {
-    const int own = pair ? wpc * 3 * (Gs + 8) : wpc * 2 * (Gs + 2), across = split ? 4 + (2 + kSplitRing) * (Gs + 8) : 0;
+    const int own = wpc * (pair ? 3 : 2) * (Gs + 8), across = split ? 4 + (2 + kSplitRing) * (Gs + 8) : 0;
     return own > across ? own : across;
 }
 
@@ -753,7 +713,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
                                                                   int min_wide, int pair_wide) {
     extern __shared__ __align__(16) float sm[];
     const int wib = threadIdx.x >> 5;
-    // rows by slot with one sentinel slot on each side (slot -1 and slot n hold +inf), Gs + 2 floats,
+    // rows by slot with one sentinel slot on each side (slot -1 and slot n hold +inf), Gs + 8 floats,
     // two per warp; then per warp a ring of the metadata of this block of 32 steps and the next one,
     // by step mod 64 (read by the narrow steps with one broadcast load); then xm (SPLIT)
     const int rows = row_floats(WPC, Gs, split != nullptr, PAIR);
@@ -786,9 +746,9 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     if (gw >= total) return;
     const int rs = __ldg(order + gw);            // longest scanlines first
     if (on && __ldg(split + 1 + scap + st.cum[rs & 15] + (rs >> 4)) >= min_wide) return;
-    float *bufA = sm + (size_t)wib * 2 * (Gs + 2) + 1;
+    float *bufA = sm + (size_t)wib * 2 * (Gs + 8) + 4;
     sgm_scanline<REC, false, 1>(cost, lo, cnt, off, H, W, P1, P2, G, agg, status, rs, mk, codes, amin, nnz_cap,
-                                bufA, bufA + (Gs + 2), meta, xm, wib);
+                                bufA, bufA + (Gs + 8), meta, xm, wib);
 }
 
 // The scanlines to split: every pixel with a window wider than 32 labels counts on its scanline of each
