@@ -40,11 +40,7 @@ PENALTY_NOTE = "P1 = 0.05 mean cost, P2 = 0.5 mean cost (coarse: per arm, intege
 
 # DRAM bytes (read + write) per launch from one ncu capture of the bench workload, with the
 # SHA-256 prefix of the kernel's source at capture time; a changed source reports null.
-NCU_TRAFFIC = {
-    "fine_cost": {"bytes": 324262400, "workload": "bench", "channels": 1,
-                  "source": "paper_1907_13449_gb300/csrc/k_fine_cost.cu",
-                  "sha256_16": "50737e8b0a1d0d04"},
-}
+NCU_TRAFFIC = {}   # no capture of the bench workload with the present row kernel (k_fine_rows.cu)
 
 
 def ncu_traffic(kernel, workload_name="bench", channels=1):
