@@ -31,7 +31,8 @@
 //
 // Colour (C = 3, Sec. III-B/C): float4 pixels (channels interleaved, 4-D tensor map) and the view's
 // three census planes; a segment holds the three channels' coefficients, a label's l2 term is the
-// Euclidean norm of its three sample differences.
+// Euclidean norm of its three sample differences.  Pixels whose differences leave the range of the fast root
+// are appended to the list.
 //
 // A pixel's costs depend on its row's own g0 only, not on the task that its row is in, and the views
 // are added in order.
@@ -221,7 +222,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3)
                    int W, int ref, const int *__restrict__ lo, const int *__restrict__ cnt,
                    const long long *__restrict__ off, const float *__restrict__ views_pad,
                    const uint64_t *__restrict__ cen_pad, float wl2, float wc, float *__restrict__ cost,
-                   int *__restrict__ status, const __grid_constant__ RowPlan pl) {
+                   int *__restrict__ status, int2 *__restrict__ list, int *__restrict__ list_count,
+                   const __grid_constant__ RowPlan pl) {
     static_assert(KW > 32 && KW <= 44 && KW % 4 == 0, "a range holds every window of at most 32 labels");
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -445,6 +447,21 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3)
     }
     if (!ok) return;                                       // (the other warps give up as well)
     if (mk == 0) continue;
+    if constexpr (C > 1) {
+        // sqrt_fast's range: a squared difference that overflows gives NaN, one below 2^-126 is off by at most
+        // 2^-63.  A pixel with a sum that is not finite, or not 0 and so small that this shows, goes to the list
+        // kernel, which runs next and takes sqrtf.  (Looking at each segment's coefficients for it: 2377 -> 2464 us
+        // on the 9x9 x 512^2 final map; here, once per pixel, within 0.1 %.)
+        bool redo = false;
+#pragma unroll
+        for (int i = 0; i < KW; i++) redo |= !(acc[i] < __int_as_float(0x7f800000)) || (acc[i] > 0.f && acc[i] < 0x1p-29f);
+        const unsigned rm = __ballot_sync(0xffffffffu, redo && on);
+        if (rm) {
+            int base = lane == 0 ? atomicAdd(list_count, __popc(rm)) : 0;
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (rm >> lane & 1) list[base + __popc(rm & ((1u << lane) - 1u))] = make_int2(y * W + x, 0);
+        }
+    }
     // a word holds d(i) + d(i+1) 2^16 (two's complement, |d| < 2^15): split it exactly
     int run = 0;
 #pragma unroll
@@ -694,7 +711,8 @@ cudaError_t launch_row_tasks(cudaStream_t s, const RowPlanHost *ph, int G, int H
 cudaError_t launch_fine_cost_rows(cudaStream_t s, const RowPlanHost *ph, const float *views_pad,
                                   const uint64_t *cen_pad, const unsigned char *desc, const int4 *heads,
                                   const RowTask *tasks, const int *extra, int G, int nviews, int H, int W, int ref, const int *lo,
-                                  const int *cnt, const long long *off, float wl2, float wc, float *cost, int *status) {
+                                  const int *cnt, const long long *off, float wl2, float wc, float *cost, int *status,
+                                  int2 *list, int *list_count) {
     RowPlan pl;
     memcpy(&pl, ph->raw, sizeof(pl));
     auto kern = pl.C == 3 ? fine_cost_rows<36, 3> : (pl.kw == 44 ? fine_cost_rows<44, 1> : fine_cost_rows<36, 1>);
@@ -705,7 +723,7 @@ cudaError_t launch_fine_cost_rows(cudaStream_t s, const RowPlanHost *ph, const f
     const int nblk = row_blocks(H, W), more = std::min(7 * nblk, std::max(nblk, 608));
     kern<<<nblk + more, 32 * kRowWarps, pl.smem, s>>>(*(const CUtensorMap *)ph->tm_v, *(const CUtensorMap *)ph->tm_c, desc,
                                                   heads, tasks, extra, nblk, G, nviews, H, W, ref, lo, cnt, off,
-                                                  views_pad, cen_pad, wl2, wc, cost, status, pl);
+                                                  views_pad, cen_pad, wl2, wc, cost, status, list, list_count, pl);
     return cudaGetLastError();
 }
 

@@ -713,7 +713,8 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
         LFSGM_TRY(run(h, "fine_cost", [&] {
             return launch_fine_cost_rows(s, &h->rows, h->views_pad, h->cen_pad, h->d_rowdesc, h->d_rowheads, h->row_tasks,
                                          h->wide_count + 1, c.fine_labels, h->nviews, c.H, c.W, h->ref, lo, cnt,
-                                         (const long long *)off, c.w_l2, c.w_census, cost, h->status);
+                                         (const long long *)off, c.w_l2, c.w_census, cost, h->status, h->wide_list,
+                                         h->wide_count);
         }));
     } else {
         // shapes whose row tiles do not fit the TMA boxes: every pixel through the list kernel

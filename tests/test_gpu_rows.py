@@ -63,3 +63,62 @@ def test_blocks_and_tasks_match_the_oracle(gpu_lib, H, W, kind, channels):
     pad = np.ones(off[-1], bool)
     pad[np.repeat(off[:-1], cnt) + np.arange(cnt.sum()) - np.repeat(np.cumsum(cnt) - cnt, cnt)] = False
     assert not np.any(got[:off[-1]][pad])                    # padding slots are 0
+
+
+def _rgb_costs(gpu_lib, p, views, lo, cnt):
+    """The colour cost volume's active slots in the row kernel and, with span 44, in the list kernel."""
+    import torch
+    off = pad4_offsets(cnt)
+    out = []
+    for kw in (36, 44):
+        L = gpu_lib.LightFieldDepth(p)
+        gpu_lib.lfsgm_set_tuning(L.h, kw)
+        L.lo.copy_(torch.from_numpy(lo))
+        L.cnt.copy_(torch.from_numpy(cnt))
+        L.off.copy_(torch.from_numpy(off))
+        L.cost_volume(torch.from_numpy(views).cuda())
+        gpu_lib.lfsgm_sync(L.h)
+        out.append(gather(L.cost.cpu().numpy(), off, cnt))
+        L.close()
+    return out
+
+
+def _rgb_case(**kw):
+    p = lfsynth.LFParams(U=3, V=4, H=9, W=37, census_w=5, dmin=-3.0, dmax=3.0, coarse_labels=16, fine_labels=121,
+                         fine_radius=7, channels=3, **kw)
+    y, x = np.mgrid[0:p.H, 0:p.W]
+    lo = (40 + (x + y) % 3).astype(np.int32).reshape(-1)
+    return p, lfsynth.random_views(p.U, p.V, p.H, p.W, seed=4, channels=3), lo, np.full(p.N, 31, np.int32)
+
+
+def test_colour_costs_of_huge_differences_are_infinite_not_nan(gpu_lib):
+    """A reference value whose squared difference overflows gives +inf (also an infinite one), a NaN NaN, and
+    1e19, whose squares' sum does not overflow, its norm; in both kernels.  The other pixels do not change."""
+    p, views, lo, cnt = _rgb_case(w_census=0.0)
+    _, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    ref = ref.reshape(p.N, 31)
+    bad = {3: 1e25, 40: -1e25, 77: np.inf, 130: -np.inf, 200: np.nan, 290: 1e19}
+    for q, v in bad.items():
+        views[p.vc, p.uc, :1 if q == 40 else 3].reshape(-1, p.N)[:, q] = v
+    for got in _rgb_costs(gpu_lib, p, views, lo, cnt):
+        got = got.reshape(p.N, 31)
+        for q, v in bad.items():
+            if np.isnan(v):
+                assert np.all(np.isnan(got[q]))
+            elif abs(v) > 1e20:
+                assert np.all(np.isposinf(got[q])), (q, v, got[q])
+            else:
+                assert np.allclose(got[q], (p.U * p.V - 1) * np.sqrt(3.0) * v, rtol=RTOL, atol=0.0)
+        same = np.setdiff1d(np.arange(p.N), list(bad))
+        assert csr_rel_err(got[same].ravel(), ref[same].ravel(), cnt[same]) <= RTOL
+
+
+# FP32 scales exactly by powers of two until a squared norm has less than 24 bits left: at 2^-63 a difference of
+# 0.01 or more of the range loses at most 2^-12 of itself, below 1e-6 of its pixel's sum
+@pytest.mark.parametrize("scale", [2.0 ** -20, 2.0 ** -50, 2.0 ** -63, 2.0 ** 50])
+def test_colour_costs_scale_with_the_views(gpu_lib, scale):
+    p, views, lo, cnt = _rgb_case(w_census=0.0)
+    views = (views * np.float32(scale)).astype(np.float32)
+    _, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    for got in _rgb_costs(gpu_lib, p, views, lo, cnt):
+        assert csr_rel_err(got, ref, cnt) <= RTOL
