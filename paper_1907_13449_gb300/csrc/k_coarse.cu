@@ -10,7 +10,7 @@
 //    shifts as linear offsets from a per-arm table.
 //  - SGM: one warp per (arm, direction, scanline), above 64 labels, or two scanlines a warp; the
 //    lane's labels stay in registers, the d-1 / d+1 neighbours across lanes come by one shuffle each
-//    way, the predecessor minimum by one redux.sync (two scanlines: two); the next 8 cost rows are
+//    way, the predecessor minimum by one redux.sync (two scanlines: two); the next 8 (7) cost rows are
 //    copied ahead into shared memory; the directions add into the sums
 //    with one packed 32/64-bit reduction per lane and step (the host checks that a label's sum
 //    over the paths stays below 2^16, so the 16-bit fields never carry into each other).
@@ -300,6 +300,10 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
     // Rows in flight, copied asynchronously into a ring per warp (a ring of registers filled by plain
     // loads waits earlier than its depth says: a warp has six scoreboards for all its loads).
     constexpr int R = 8;
+    // Two-byte rows, which even lanes copy for their odd neighbours too: one row less, so that a step refills
+    // the slot of the step before it, which both lanes have read before this step's __syncwarp (3x3 x 376 x 541, 32
+    // labels: host to host 587 us, with eight rows and a second __syncwarp a step 600).
+    constexpr int D = sizeof(T) == 2 ? R - 1 : R;
     __shared__ __align__(16) T cring[4][R][32];
     constexpr uint32_t SENT = 0x7fff7fffu;
     const int lane = threadIdx.x & 31, gl = lane & (GL - 1), wib = threadIdx.x >> 5;
@@ -366,7 +370,7 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
             words_of<LPT>(v, c);
         }
     };
-    for (int i = 0; i < R; i++) ld(i, i < steps);
+    for (int i = 0; i < D; i++) ld(i, i < steps);
     uint32_t L[NP];
     uint32_t mm = 0;                                                 // (m, m)
     auto finish = [&](const uint32_t *Ln, bool on) {   // group minimum, packed reduction, carry the row
@@ -386,13 +390,14 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
 #pragma unroll
         for (int j = 0; j < NP; j++) L[j] = Ln[j];
     };
-    // one step on the row in ring slot i (the oldest copy), whose slot then takes the row R steps on
+    // one step on the row in ring slot i (the oldest copy); the row D steps on is requested
     auto step = [&](int i, bool start, bool in, bool on) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(R - 1) : "memory");
+        asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
         if constexpr (sizeof(T) == 2) __syncwarp();
         uint32_t c[NP];
-        words(cring[wib][i][lane], c);
-        ld(i, in);
+        const T v = cring[wib][i][lane];
+        ld((i + D) & (R - 1), in);
+        words(v, c);
         if (start) {   // path start: L = C
             finish(c, on);
             return;
@@ -416,14 +421,14 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
         }
         finish(Ln, on);
     };
-    step(0, true, R < steps, have);
+    step(0, true, D < steps, have);
     // R steps at a time, as long as both groups have all of them and the rows to load; then the rest
     int t0 = 1;
     for (; t0 + 2 * R <= least; t0 += R) {
 #pragma unroll
         for (int k = 0; k < R; k++) step((1 + k) & (R - 1), false, true, true);   // (t0 = 1 mod R)
     }
-    for (int t = t0; t < most; t++) step(t & (R - 1), false, t + R < steps, SUB == 1 || t < steps);
+    for (int t = t0; t < most; t++) step(t & (R - 1), false, t + D < steps, SUB == 1 || t < steps);
 }
 
 // WTA over the path sums (Eq. 10): lowest label on ties (the key is sum << 8 | label).

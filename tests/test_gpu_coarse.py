@@ -27,3 +27,23 @@ def test_coarse_maps_match_the_oracle(gpu_lib, Lc, U, V, H, W, paths):
     assert np.array_equal(L.maps.cpu().numpy()[:n], np.asarray(ref["maps"]).reshape(n, -1))
     assert np.array_equal(L.lo.cpu().numpy(), ref["lo"]) and np.array_equal(L.cnt.cpu().numpy(), ref["cnt"])
     L.close()
+
+
+# byte rows of two labels a lane (up to 32 labels), whose copies even lanes make for their odd neighbours: scanlines
+# of many times the rows in flight, odd label counts, the same maps every time
+@pytest.mark.parametrize("Lc", [3, 17, 30, 32])
+@pytest.mark.parametrize("H,W,paths", [(33, 301, 8), (257, 19, 16)])
+def test_copied_byte_rows_match_the_oracle_each_time(gpu_lib, Lc, H, W, paths):
+    import torch
+    p = lfsynth.LFParams(U=3, V=3, H=H, W=W, census_w=5, dmin=-1.5, dmax=1.5, coarse_labels=Lc, fine_labels=31,
+                         fine_radius=4, paths=paths)
+    views = lfsynth.random_views(3, 3, H, W, seed=Lc + W)
+    ref = oracle.initial_disparity(oracle.make_cfg(p), views, p1f=p.p1_frac, p2f=p.p2_frac)
+    L = gpu_lib.LightFieldDepth(p)
+    n = len(ref["arms"])
+    for _ in range(4):
+        L.maps.fill_(-1)
+        L.initial(torch.from_numpy(views).cuda())
+        gpu_lib.lfsgm_sync(L.h)
+        assert np.array_equal(L.maps.cpu().numpy()[:n], np.asarray(ref["maps"]).reshape(n, -1))
+    L.close()
