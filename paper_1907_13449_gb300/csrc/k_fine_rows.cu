@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3)
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned mbar = smem_u32(smem + pl.o_mbar);      // full[stages] at +0, empty[stages] at +64
+    volatile int *gave_up = (volatile int *)(smem + pl.o_mbar + 120);   // a warp's wait has expired
     const int S = pl.stages, ls = S == 4 ? 2 : 1;          // a power of two: view vi uses stage vi mod S
     // a CTA per block and per further task; more than that (the rows of many blocks differ) in turn
     bool inited = false;
@@ -247,8 +248,12 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3)
     const int nv = nviews - 1;                             // the views without the reference
     int4 *hds = (int4 *)(smem + pl.o_hd);
     unsigned char *nbs = smem + pl.o_nb;
-    if (inited) __syncthreads();              // every warp is done with the previous task
+    if (inited) {
+        __syncthreads();                      // every warp is done with the previous task
+        if (*gave_up) return;                 // all of them: the barriers of a warp that gave up are not set up anew
+    }
     if (threadIdx.x == 0) {
+        if (!inited) *gave_up = 0;
         for (int s = 0; s < S; s++) {
             if (inited) {
                 asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(mbar + 8 * s) : "memory");
@@ -441,12 +446,14 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3)
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar + 64 + 8 * st) : "memory");
     }
     if (!ok) {
-        if (lane == 0) atomicExch(status, 6);
+        if (lane == 0) {
+            atomicExch(status, 6);
+            *gave_up = 1;
+        }
         // let the copies still in flight land (bounded) before the CTA's shared memory is released
         for (int v = vi; v < min(nv, vi + S); v++) mbar_wait(mbar + 8 * (v & (S - 1)), (unsigned)(v >> ls) & 1u);
     }
-    if (!ok) return;                                       // (the other warps give up as well)
-    if (mk == 0) continue;
+    if (!ok || mk == 0) continue;                          // (to the barrier above)
     if constexpr (C > 1) {
         // sqrt_fast's range: a squared difference that overflows gives NaN, one below 2^-126 is off by at most
         // 2^-63.  A pixel with a sum that is not finite, or not 0 and so small that this shows, goes to the list

@@ -122,3 +122,30 @@ def test_colour_costs_scale_with_the_views(gpu_lib, scale):
     _, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
     for got in _rgb_costs(gpu_lib, p, views, lo, cnt):
         assert csr_rel_err(got, ref, cnt) <= RTOL
+
+
+# more tasks than CTAs: rows of eight different spans in each of 175 blocks (1400 tasks, 783 CTAs), so that a CTA
+# runs a second task on barriers set up anew, with rows that have no pixel in it
+@pytest.mark.parametrize("channels", [1, 3])
+def test_more_tasks_than_ctas_match_the_oracle(gpu_lib, channels):
+    import torch
+    H = W = 200
+    p = lfsynth.LFParams(U=3, V=4, H=H, W=W, census_w=5, dmin=-3.0, dmax=3.0, coarse_labels=16, fine_labels=441,
+                         fine_radius=7, channels=channels)
+    rng = np.random.default_rng(7 + channels)
+    views = lfsynth.random_views(p.U, p.V, H, W, seed=11, channels=channels)
+    y = np.repeat(np.arange(H), W)
+    lo = ((y % 8) * 52 + rng.integers(0, 3, H * W)).astype(np.int32)    # starts at least 50 apart: a task a row
+    cnt = rng.integers(5, 29, H * W).astype(np.int32)
+    off = pad4_offsets(cnt)
+    L = gpu_lib.LightFieldDepth(p)
+    L.lo.copy_(torch.from_numpy(lo))
+    L.cnt.copy_(torch.from_numpy(cnt))
+    L.off.copy_(torch.from_numpy(off))
+    off_o, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    for _ in range(2):
+        L.cost.fill_(float("nan"))
+        L.cost_volume(torch.from_numpy(views).cuda())
+        gpu_lib.lfsgm_sync(L.h)
+        assert csr_rel_err(gather(L.cost.cpu().numpy(), off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
+    L.close()
