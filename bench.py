@@ -242,7 +242,7 @@ def run_ours(args, ws, rank, local):
     if args.sgm_warps is not None or args.sgm_split is not None:
         knob_note += "; SGM knobs fixed on the command line"
     sgm_warps = lf.lfsgm_get_tuning(L.h)[2]
-    sgm_split = lf.lfsgm_get_sgm_split(L.h)
+    sgm_split = lf.lfsgm_sgm_split_used(L.h)
 
     def step(events=None):
         L.initial(views)

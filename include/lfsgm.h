@@ -127,16 +127,19 @@ lfsgm_status lfsgm_get_tuning(lfsgm_handle h, int32_t *row_kw, int32_t *list_cta
 
 /* Speed knob of the fine SGM (not in the paper): a scanline that crosses at least min_wide
  * windows wider than 32 labels runs on all the warps of one CTA, which share each wide step's
- * 32-label chunks, instead of on one warp.  0, the default: 24 for images of at least 256 pixels in a
- * direction, none for smaller ones and for searches over the whole range.  Such
+ * labels, four to a thread, instead of on one warp (0: none does, and every scanline has a warp of
+ * its own).  While it is not set, the library takes 24 for images of at least 256 pixels in a
+ * direction, and none for smaller ones and for searches over the whole range.  Such
  * scanlines (along image borders, where the initial pass leaves whole-range windows) otherwise
  * outlast all others; the CTA's other warps wait while its first runs the narrow steps, so the
  * split pays only where a few scanlines are much longer than the rest.  The kernel that clears agg
  * lists them; when more than 256 qualify (most windows wide), none is split.  The aggregate is the
- * same bit for bit with any value (a large one: none).  lfsgm_get_sgm_split reads it back.
- * Errors: LFSGM_ERR_INVALID_ARG for a negative value. */
+ * same bit for bit with any value.  lfsgm_get_sgm_split reads back what the caller or lfsgm_autotune
+ * has set (0 also while nothing is set), lfsgm_sgm_split_used the threshold that the calls run with
+ * (0: none).  Errors: LFSGM_ERR_INVALID_ARG for a negative value. */
 lfsgm_status lfsgm_set_sgm_split(lfsgm_handle h, int32_t min_wide);
 lfsgm_status lfsgm_get_sgm_split(lfsgm_handle h, int32_t *min_wide);
+lfsgm_status lfsgm_sgm_split_used(lfsgm_handle h, int32_t *min_wide);
 
 /* Picks the speed knobs for this handle's shape on a representative light field (views: device,
  * as for lfsgm_depth): one initial pass, then the cost stage is timed with the row kernel's label
@@ -144,7 +147,8 @@ lfsgm_status lfsgm_get_sgm_split(lfsgm_handle h, int32_t *min_wide);
  * kernel's CTAs per SM 8, 12 and 24
  * against the default; the fastest setting is kept (lfsgm_set_tuning) and returned in row_kw and
  * list_ctas_per_sm (host, nullable).  Then lfsgm_sgm_aggregate (derived penalties) is timed with
- * 4, 8 and 2 SGM warps per CTA and the fastest kept (lfsgm_set_sgm_warps; lfsgm_get_tuning).
+ * 4, 8 and 2 SGM warps per CTA, each with split threshold 24 and without split, and the fastest pair
+ * kept (lfsgm_set_sgm_warps, lfsgm_set_sgm_split).
  * Synchronous; uses the buffers of lfsgm_depth. */
 lfsgm_status lfsgm_autotune(lfsgm_handle h, const float *views, int32_t *row_kw, int32_t *list_ctas_per_sm);
 

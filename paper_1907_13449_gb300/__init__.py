@@ -67,7 +67,7 @@ EXPORTS = ["lfsgm_create", "lfsgm_destroy", "lfsgm_workspace_size", "lfsgm_set_w
            "lfsgm_batch_destroy", "lfsgm_median_filter", "lfsgm_batch_workspace_size", "lfsgm_batch_create_ws",
            "lfsgm_set_tuning", "lfsgm_batch_knobs", "lfsgm_autotune", "lfsgm_sgm_aggregate_record",
            "lfsgm_backward_recorded", "lfsgm_set_sgm_warps", "lfsgm_get_tuning", "lfsgm_batch_sgm_warps",
-           "lfsgm_set_sgm_split", "lfsgm_get_sgm_split", "lfsgm_batch_sgm_split"]
+           "lfsgm_set_sgm_split", "lfsgm_get_sgm_split", "lfsgm_sgm_split_used", "lfsgm_batch_sgm_split"]
 
 
 def load(build_if_missing: bool = False):
@@ -100,6 +100,7 @@ def load(build_if_missing: bool = False):
         L.lfsgm_set_sgm_warps.argtypes = [vp, i32]
         L.lfsgm_set_sgm_split.argtypes = [vp, i32]
         L.lfsgm_get_sgm_split.argtypes = [vp, C.POINTER(i32)]
+        L.lfsgm_sgm_split_used.argtypes = [vp, C.POINTER(i32)]
         L.lfsgm_get_tuning.argtypes = [vp, P(i32), P(i32), P(i32)]
         L.lfsgm_batch_sgm_warps.argtypes = [vp, vp]
         L.lfsgm_batch_sgm_split.argtypes = [vp, vp]
@@ -404,15 +405,22 @@ def lfsgm_set_sgm_warps(h, warps_per_cta=0):
 
 def lfsgm_set_sgm_split(h, min_wide=0):
     """Speed knob of the fine SGM: scanlines crossing at least min_wide windows wider than 32
-    labels run on all warps of a CTA (0: 24 for images of 256 pixels or more in a direction, unless
-    every window is the whole range; a large value: none)."""
+    labels run on all warps of a CTA (0: none does).  While it is not set: 24 for images of 256
+    pixels or more in a direction, unless every window is the whole range."""
     _check(load().lfsgm_set_sgm_split(h, int(min_wide)), h)
 
 
 def lfsgm_get_sgm_split(h):
-    """The handle's SGM split threshold (0: off)."""
+    """The SGM split threshold that was set on the handle (0: off, or none set)."""
     v = C.c_int32()
     _check(load().lfsgm_get_sgm_split(h, C.byref(v)), h)
+    return int(v.value)
+
+
+def lfsgm_sgm_split_used(h):
+    """The SGM split threshold that the handle's calls run with (0: none is split)."""
+    v = C.c_int32()
+    _check(load().lfsgm_sgm_split_used(h, C.byref(v)), h)
     return int(v.value)
 
 
@@ -432,7 +440,7 @@ def lfsgm_batch_sgm_warps(b, n):
 
 
 def lfsgm_batch_sgm_split(b, n):
-    """The fine SGM's split threshold of each light field of a batch (numpy int32 array; 0: off)."""
+    """The fine SGM's split threshold that each light field of a batch runs with (numpy int32 array; 0: off)."""
     import numpy as np
     w = np.zeros(n, np.int32)
     _bcheck(load().lfsgm_batch_sgm_split(b, w.ctypes.data_as(C.c_void_p)), b)

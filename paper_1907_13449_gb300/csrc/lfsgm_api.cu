@@ -61,8 +61,8 @@ struct lfsgm_ctx {
     // tuning knobs (lfsgm_set_tuning): label span of the row kernel's ranges, list-kernel CTAs per SM
     int row_kw = 36, list_ctas = 0, sgm_warps = 4;
     // scanlines that cross at least this many windows wider than 32 labels run split across a CTA's
-    // warps (lfsgm_set_sgm_split; 0: see split_from)
-    int sgm_split = 0;
+    // warps (lfsgm_set_sgm_split; 0: none, -1: not set, see split_from)
+    int sgm_split = -1;
     std::vector<FineTap> h_fine;          // host copy of the shift table (row descriptors are rebuilt from it)
     // device tables
     FineTap *d_fine = nullptr;
@@ -253,6 +253,18 @@ lfsgm_status ensure_workspace(lfsgm_ctx *h) {
 // whose samples could make 0 x l2 a NaN (flagged with the census).
 bool census_only(const lfsgm_ctx *h) { return h->cfg.w_l2 == 0.f && h->C == 1; }
 int *large_flag(lfsgm_ctx *h) { return census_only(h) ? h->wide_count + 2 : nullptr; }
+
+// Windows wider than 32 labels from which on a scanline runs split across a CTA (0: none does).  Where
+// the caller has set no threshold: 24, unless scanlines are short (a scanline of 256 steps with 24 such
+// windows takes about as long as one of 340 without) or every window is the whole range (then all are
+// alike).  Two scanlines of 9x9 x 512^2 cross 147 windows of 401 labels each and outlast all others:
+// 297 us without, 242 with the split (24, 48 and 96 alike, 215 with vectors of four labels; recording 382
+// and 313); the same time without such scanlines.  8 or 12 list more than the table holds.
+int split_from(const lfsgm_ctx *h) {
+    const lfsgm_config &c = h->cfg;
+    if (h->sgm_split >= 0) return h->sgm_split;
+    return !c.boundless && std::max(c.H, c.W) >= 256 ? 24 : 0;
+}
 
 int max_arm_views(const lfsgm_ctx *h) {
     int m = 0;
@@ -585,7 +597,13 @@ lfsgm_status lfsgm_set_sgm_split(lfsgm_handle h, int32_t min_wide) {
 
 lfsgm_status lfsgm_get_sgm_split(lfsgm_handle h, int32_t *min_wide) {
     if (!h || !min_wide) return LFSGM_ERR_INVALID_ARG;
-    *min_wide = h->sgm_split;
+    *min_wide = std::max(h->sgm_split, 0);
+    return LFSGM_OK;
+}
+
+lfsgm_status lfsgm_sgm_split_used(lfsgm_handle h, int32_t *min_wide) {
+    if (!h || !min_wide) return LFSGM_ERR_INVALID_ARG;
+    *min_wide = split_from(h);
     return LFSGM_OK;
 }
 
@@ -753,17 +771,6 @@ lfsgm_status lfsgm_cost_volume(lfsgm_handle h, const float *views, const int32_t
 }  // extern "C"
 
 namespace {
-// Windows wider than 32 labels from which on a scanline runs split across a CTA (0: none does).  Where
-// the caller has set no threshold: 24, unless scanlines are short (a scanline of 256 steps with 24 such
-// windows takes about as long as one of 340 without) or every window is the whole range (then all are
-// alike).  Two scanlines of 9x9 x 512^2 cross 147 windows of 401 labels each and outlast all others:
-// 297 us without, 242 with the split (24, 48 and 96 alike, 215 with vectors of four labels; recording 382
-// and 313); the same time without such scanlines.  8 or 12 list more than the table holds.
-int split_from(const lfsgm_ctx *h) {
-    const lfsgm_config &c = h->cfg;
-    if (h->sgm_split > 0) return h->sgm_split;
-    return !c.boundless && std::max(c.H, c.W) >= 256 ? 24 : 0;
-}
 // The split table cleared for the launch that lists the scanlines.
 lfsgm_status clear_split(lfsgm_ctx *h) {
     if (split_from(h) == 0) return LFSGM_OK;
@@ -1110,29 +1117,34 @@ lfsgm_status tune_handle(lfsgm_handle h, const float *views, int32_t *lo, int32_
     if (st == LFSGM_OK) st = lfsgm_set_tuning(h, best_kw, best_lc);
     // the SGM's warps (scanlines) per CTA, on the cost volume of the chosen knobs (derived penalties)
     if (st == LFSGM_OK) st = cost_volume_impl(h, views, lo, cnt, off, cost, !h->cfg.boundless);
-    int best_w = 4;
+    // and whether scanlines that cross many wide windows run split across a CTA (threshold 24, or none)
+    int best_w = 4, best_sp = 24;
     float best_sgm = 1e30f;
-    for (int w : {4, 8, 2}) {
-        if (st != LFSGM_OK) break;
-        st = lfsgm_set_sgm_warps(h, w);
-        float best = 1e30f;
-        for (int r = 0; r < 3 && st == LFSGM_OK; r++) {
-            cudaEventRecord(e0, h->stream);
-            st = lfsgm_sgm_aggregate(h, cost, lo, cnt, off, -1.f, -1.f, agg);
-            cudaEventRecord(e1, h->stream);
-            cudaEventSynchronize(e1);
-            float t = 0.f;
-            cudaEventElapsedTime(&t, e0, e1);
-            if (r > 0) best = std::min(best, t);
+    for (int w : {4, 8, 2})
+        for (int sp : {24, 0}) {
+            if (st != LFSGM_OK) break;
+            st = lfsgm_set_sgm_warps(h, w);
+            if (st == LFSGM_OK) st = lfsgm_set_sgm_split(h, sp);
+            float best = 1e30f;
+            for (int r = 0; r < 3 && st == LFSGM_OK; r++) {
+                cudaEventRecord(e0, h->stream);
+                st = lfsgm_sgm_aggregate(h, cost, lo, cnt, off, -1.f, -1.f, agg);
+                cudaEventRecord(e1, h->stream);
+                cudaEventSynchronize(e1);
+                float t = 0.f;
+                cudaEventElapsedTime(&t, e0, e1);
+                if (r > 0) best = std::min(best, t);
+            }
+            if (st == LFSGM_OK && best < best_sgm) {
+                best_sgm = best;
+                best_w = w;
+                best_sp = sp;
+            }
         }
-        if (st == LFSGM_OK && best < best_sgm) {
-            best_sgm = best;
-            best_w = w;
-        }
-    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st == LFSGM_OK) st = lfsgm_set_sgm_warps(h, best_w);
+    if (st == LFSGM_OK) st = lfsgm_set_sgm_split(h, best_sp);
     kw_out = best_kw;
     lc_out = best_lc;
     return st;
@@ -1670,7 +1682,7 @@ lfsgm_status lfsgm_batch_sgm_warps(lfsgm_batch b, int32_t *warps_per_cta) {
 
 lfsgm_status lfsgm_batch_sgm_split(lfsgm_batch b, int32_t *min_wide) {
     if (!b || !min_wide) return LFSGM_ERR_INVALID_ARG;
-    for (int i = 0; i < b->n; i++) min_wide[i] = b->h[i]->sgm_split;
+    for (int i = 0; i < b->n; i++) min_wide[i] = split_from(b->h[i]);
     return LFSGM_OK;
 }
 

@@ -105,3 +105,49 @@ def test_split_scanlines_record_the_adjoints_branches(gpu_lib, H, W, G):
     tol = grad_tol(_cs_max(p, lo, cnt, off_o, cost_o, P1, P2), p.softmin_tau)
     assert np.mean(eC > tol) <= 1e-4 and np.mean(eV > tol) <= 1e-4
     assert np.abs(gC - gC_o).sum() <= 1e-3 * np.abs(gC_o).sum()
+
+
+# the threshold: the library's own on a new handle (24 from 256 pixels in a direction on, not for whole-range searches),
+# 0 for none, the caller's or the autotuner's; lfsgm_get_sgm_split reads back what was set
+@pytest.mark.parametrize("H,W,boundless,own", [(20, 256, 0, 24), (256, 20, 0, 24), (255, 255, 0, 0), (20, 300, 1, 0)])
+def test_split_threshold_in_use(gpu_lib, H, W, boundless, own):
+    import torch
+    p = lfsynth.LFParams(U=3, V=3, H=H, W=W, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=40, fine_labels=75,
+                         fine_radius=5, boundless=boundless)
+    h = gpu_lib.lfsgm_create(p)
+    assert gpu_lib.lfsgm_get_sgm_split(h) == 0 and gpu_lib.lfsgm_sgm_split_used(h) == own
+    for n in (0, 24, 7, 0):
+        gpu_lib.lfsgm_set_sgm_split(h, n)
+        assert gpu_lib.lfsgm_get_sgm_split(h) == n and gpu_lib.lfsgm_sgm_split_used(h) == n
+    gpu_lib.lfsgm_set_sgm_split(h, 5)
+    gpu_lib.lfsgm_autotune(h, _dev(lfsynth.random_views(3, 3, H, W, seed=H)))
+    assert gpu_lib.lfsgm_get_sgm_split(h) == gpu_lib.lfsgm_sgm_split_used(h) and gpu_lib.lfsgm_get_sgm_split(h) in (0, 24)
+    gpu_lib.lfsgm_destroy(h)
+    v = torch.from_numpy(lfsynth.random_views(3, 3, H, W, seed=H)).cuda()
+    b = gpu_lib.LightFieldBatch([p, p], [v, v], branches=1)
+    assert b.knobs()[3].tolist() == [own, own]
+    b.close()
+
+
+# a new handle (two scanlines a warp, split from 24 on) against no split, one scanline a warp
+@pytest.mark.parametrize("H,W,rows,cols", [(20, 256, [0, 7], [3]), (256, 17, [30], [16]), (40, 256, [], list(range(20, 43))),
+                                           (300, 260, [0], []), (300, 260, range(0, 280), [])])
+@pytest.mark.parametrize("penalties", [(-1.0, -1.0), (1.5, 9.0)])
+def test_new_handle_gives_the_bits_of_no_split(gpu_lib, H, W, rows, cols, penalties):
+    import torch
+    G = 75
+    lo, cnt, off, cost = _windows(H, W, G, H + W, [r for r in rows if r < H], cols)
+    p = lfsynth.LFParams(U=3, V=3, H=H, W=W, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=40, fine_labels=G,
+                         fine_radius=5)
+    d = [_dev(cost), _dev(lo, torch.int32), _dev(cnt, torch.int32), _dev(off)]
+    h = gpu_lib.lfsgm_create(p)
+    out = []
+    for min_wide in (None, 0, 24, 1 << 30, 0):
+        if min_wide is not None:
+            gpu_lib.lfsgm_set_sgm_split(h, min_wide)
+        agg = torch.full_like(d[0], float("nan"))
+        gpu_lib.lfsgm_sgm_aggregate(h, *d, *penalties, agg)
+        out.append(agg)
+    gpu_lib.lfsgm_sync(h)
+    gpu_lib.lfsgm_destroy(h)
+    assert all(torch.equal(out[0], a) for a in out[1:])
