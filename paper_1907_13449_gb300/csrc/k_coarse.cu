@@ -395,9 +395,8 @@ __global__ void __launch_bounds__(128) coarse_sgm_kernel(const void *__restrict_
         asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
         if constexpr (sizeof(T) == 2) __syncwarp();
         uint32_t c[NP];
-        const T v = cring[wib][i][lane];
+        words(cring[wib][i][lane], c);
         ld((i + D) & (R - 1), in);
-        words(v, c);
         if (start) {   // path start: L = C
             finish(c, on);
             return;
