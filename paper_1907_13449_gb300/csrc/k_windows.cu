@@ -186,7 +186,9 @@ __global__ void __launch_bounds__(256) fused_windows_kernel(const int *__restric
                                                             double phi, int passes, WindowArgs a) {
     constexpr int TW = 36, TH = 12;
     __shared__ int t[2][TH][TW];
-    const int x0 = blockIdx.x * 32 - passes, y0 = blockIdx.y * 8 - passes;   // image position of tile entry (0, 0)
+    const int bx = (W + 31) >> 5, by = blockIdx.x / bx;                      // (one grid dimension: images of any height)
+    const int xt = (blockIdx.x - by * bx) * 32, yt = by * 8;                 // the tile
+    const int x0 = xt - passes, y0 = yt - passes;                            // image position of entry (0, 0)
     const int tid = threadIdx.y * 32 + threadIdx.x;
     for (int i = tid; i < TW * TH; i += 256) {
         const int ty = i / TW, tx = i - ty * TW, x = x0 + tx, y = y0 + ty;
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(256) fused_windows_kernel(const int *__restric
         }
         __syncthreads();
     }
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+    const int x = xt + threadIdx.x, y = yt + threadIdx.y;
     const bool in = x < W && y < H;
     int pad = 0;
     if (in) pad = window_of(a, y * W + x, x, y, t[passes & 1][threadIdx.y + passes][threadIdx.x + passes]);
@@ -301,8 +303,8 @@ cudaError_t launch_windows(cudaStream_t s, const int *F, int N, int W, const Win
 }
 cudaError_t launch_fused_windows(cudaStream_t s, const int *maps, int narms, int H, int W, double phi, int passes,
                                  const WindowSetup &u) {
-    fused_windows_kernel<<<dim3((W + 31) / 32, (H + 7) / 8), dim3(32, 8), 0, s>>>(maps, narms, H, W, phi, passes,
-                                                                                 window_args(u));
+    fused_windows_kernel<<<(W + 31) / 32 * ((H + 7) / 8), dim3(32, 8), 0, s>>>(maps, narms, H, W, phi, passes,
+                                                                              window_args(u));
     return cudaGetLastError();
 }
 int scan_tiles(int N) { return (N + kScanTile - 1) / kScanTile; }

@@ -52,3 +52,24 @@ def test_offsets_are_the_padded_counts_prefix_sums(gpu_lib, H, W):
     gpu_lib.lfsgm_destroy(h)
     assert len(np.unique(_np(cnt))) > 1
     assert np.array_equal(_np(off), pad4_offsets(_np(cnt)))
+
+
+# taller than 65535 tiles of eight rows: the windows of a column of views and of its transpose, a row
+def test_windows_of_a_very_tall_image_are_its_transposes(gpu_lib):
+    import torch
+    N = 8 * 65535 + 9
+    views = np.random.default_rng(5).random((2, N)).astype(np.float32)
+    got = []
+    for U, V, H, W in ((1, 2, N, 1), (2, 1, 1, N)):
+        p = lfsynth.tiny_params(U=U, V=V, H=H, W=W, coarse_labels=33, fine_labels=21, fill_passes=2, phi=1.0)
+        lo = torch.empty(N, dtype=torch.int32, device="cuda")
+        cnt = torch.empty_like(lo)
+        off = torch.empty(N + 1, dtype=torch.int64, device="cuda")
+        h = gpu_lib.lfsgm_create(p)
+        gpu_lib.lfsgm_initial_disparity(h, _dev(views.reshape(V, U, H, W)), 0, 0, lo, cnt, off, None, None)
+        gpu_lib.lfsgm_sync(h)
+        gpu_lib.lfsgm_destroy(h)
+        got.append((_np(lo), _np(cnt), _np(off)))
+    assert len(np.unique(got[0][0])) > 1 and np.array_equal(got[0][2], pad4_offsets(got[0][1]))
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
