@@ -530,15 +530,18 @@ bool plan_fine_rows(int U, int V, int uc, int vc, int H, int W, int G, double dm
     pl.Hp = H + 2 * pl.P;
     const double step = (dmax - dmin) / (double)(G - 1);
     const int ax = std::max(uc, U - 1 - uc), ay = std::max(vc, V - 1 - vc);
-    const int kwt = kRowKW + 4;                          // a task spans 4 labels more than a row's range
-    pl.kwt = kwt;
-    const int spx = (int)ceil(ax * step * (kwt - 1)), spy = (int)ceil(ay * step * (kwt - 1));
-    // taps: columns x0+oxlo .. x0+32+oxhi, rows y0+oylo .. y0+7+oyhi+1, with oxhi-oxlo <= spx, one label of
-    // slack below the FP32 origin estimate and up to 3 (floats) / 1 (words) columns of 16-byte rounding
-    pl.bwf = (spx + 38 + 3) & ~3;
-    pl.bhf = spy + 4 + kBlkH - 1;
-    pl.bwc = (spx + 35 + 1) & ~1;
-    pl.bhc = spy + 3 + kBlkH - 1;
+    // a task spans 4 labels more than a row's range, or, where a box would then be too large for TMA, none
+    for (int more = 4; more >= 0; more -= 4) {
+        pl.kwt = kRowKW + more;
+        const int spx = (int)ceil(ax * step * (pl.kwt - 1)), spy = (int)ceil(ay * step * (pl.kwt - 1));
+        // taps: columns x0+oxlo .. x0+32+oxhi, rows y0+oylo .. y0+7+oyhi+1, with oxhi-oxlo <= spx, one label of
+        // slack below the FP32 origin estimate and up to 3 (floats) / 1 (words) columns of 16-byte rounding
+        pl.bwf = (spx + 38 + 3) & ~3;
+        pl.bhf = spy + 4 + kBlkH - 1;
+        pl.bwc = (spx + 35 + 1) & ~1;
+        pl.bhc = spy + 3 + kBlkH - 1;
+        if (pl.bwf <= 256 && pl.bwc <= 256 && pl.bhf <= 256 && pl.bhc <= 256) break;
+    }
     pl.seg_cap = std::min(kRowKW, (int)ceil(ax * step * (kRowKW - 1)) + (int)ceil(ay * step * (kRowKW - 1)) + 3);
     pl.ds_stride = (kDsSegs + pl.seg_cap * (kDsSegBytes + kDsCenBytes) + 15) & ~15;
     pl.o_rc = r128(pl.bwf * pl.bhf * 4 * (C == 1 ? 1 : 4));               // colour: float4 pixels

@@ -149,3 +149,31 @@ def test_more_tasks_than_ctas_match_the_oracle(gpu_lib, channels):
         gpu_lib.lfsgm_sync(L.h)
         assert csr_rel_err(gather(L.cost.cpu().numpy(), off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
     L.close()
+
+
+def test_ranges_whose_boxes_just_fit_take_the_row_kernel(gpu_lib):
+    """A range of 36 labels over 200 pixels (a row of nine views): 40 labels would not fit a 256-wide box, so tasks
+    span the 36 labels of a row's own range."""
+    import torch
+    G = 81
+    p = lfsynth.LFParams(U=9, V=1, H=19, W=97, census_w=5, dmin=-57.0, dmax=57.0, coarse_labels=16, fine_labels=G,
+                         fine_radius=7)
+    rng = np.random.default_rng(3)
+    views = lfsynth.random_views(p.U, p.V, p.H, p.W, seed=2)
+    lo = rng.integers(0, G, p.N).astype(np.int32)
+    lo[:p.N // 2] = 20 + lo[:p.N // 2] % 5
+    cnt = np.minimum(rng.integers(5, 33, p.N), G - lo).astype(np.int32)
+    off = pad4_offsets(cnt)
+    L = gpu_lib.LightFieldDepth(p)
+    L.lo.copy_(torch.from_numpy(lo))
+    L.cnt.copy_(torch.from_numpy(cnt))
+    L.off.copy_(torch.from_numpy(off))
+    vd = torch.from_numpy(views).cuda()
+    gpu_lib.lfsgm_set_profiling(L.h, True)
+    L.cost_volume(vd)
+    gpu_lib.lfsgm_sync(L.h)
+    assert "row_tasks" in [n for n, _ in gpu_lib.lfsgm_kernel_times(L.h)]
+    got = L.cost.cpu().numpy()
+    L.close()
+    off_o, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    assert csr_rel_err(gather(got, off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
