@@ -43,6 +43,18 @@ PENALTY_NOTE = "P1 = 0.05 mean cost, P2 = 0.5 mean cost (coarse: per arm, intege
 NCU_TRAFFIC = {}   # no capture of the bench workload with the present row kernel (k_fine_rows.cu)
 
 
+# The kernels of the cost and SGM stages (derived penalties), by their names in lfsgm_kernel_times.
+COST_SGM_KERNELS = ["census_all", "census_rest", "row_tasks", "fine_cost", "fine_cost_all_list", "fine_cost_runs",
+                    "fine_cost_census", "fine_cost_wide", "cost_partial_sums", "fine_sgm"]
+
+
+def dominant_kernel(kernels):
+    """The cost or SGM kernel with the most time.  A grey volume without the l2 term (fine_cost_census) leaves the
+    list kernel (fine_cost_wide) nothing to do."""
+    skip = {"fine_cost_wide"} if "fine_cost_census" in kernels else set()
+    return max((k for k in kernels if k in COST_SGM_KERNELS and k not in skip), key=lambda k: kernels[k]["ms_total"])
+
+
 def ncu_traffic(kernel, workload_name="bench", channels=1):
     import hashlib
     e = NCU_TRAFFIC.get(kernel)
@@ -363,10 +375,9 @@ def run_ours(args, ws, rank, local):
     K = args.steps
     value = ms_per_lf(stage_ms, K, ws)          # whole-job ms per light field (cost+SGM)
     # dominant kernel of the cost+SGM stages and its roofline
-    hot = ["fine_cost", "fine_cost_wide", "fine_sgm", "census_all", "cost_partial_sums", "zero_agg", "sgm_split"]
     if "fine_cost" not in kernels:
         row_cells = 0                     # no row-kernel plan for this shape: every window in the list
-    dom = max((k for k in kernels if k in hot), key=lambda k: kernels[k]["ms_total"])
+    dom = dominant_kernel(kernels)
     mhz = (clocks or {}).get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     by = hbm_bytes_cost_sgm(p, active)

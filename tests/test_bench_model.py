@@ -30,3 +30,20 @@ def test_row_kernel_cells_prefers_the_lowest_start_on_ties():
     cnt[0] = 20                                     # a narrower window in the start-40 group
     got = bench.row_kernel_cells(lo, cnt, 1, 32)
     assert got == 16 * 31
+
+
+def test_dominant_kernel_is_among_the_kernels_the_stages_launch():
+    import os
+    import re
+    api = open(os.path.join(os.path.dirname(bench.__file__), "paper_1907_13449_gb300", "csrc", "lfsgm_api.cu")).read()
+
+    def launched(start, end):
+        return set(re.findall(r'run\(h, "(\w+)"', api[api.index(start):api.index(end)]))
+    stages = launched("lfsgm_status cost_volume_impl(", "\nint *split_table") | launched("lfsgm_status lfsgm_sgm_aggregate(", "lfsgm_status lfsgm_wta_subpixel(")
+    assert set(bench.COST_SGM_KERNELS) == stages - {"set_penalties"}    # (explicit penalties only)
+    ms = dict(census_all=0.03, fine_cost=0.01, fine_cost_runs=0.17, fine_cost_census=0.02, fine_cost_wide=0.2, fine_sgm=0.1,
+              coarse_sgm=0.5)
+    kernels = {k: {"ms_total": v} for k, v in ms.items()}
+    assert bench.dominant_kernel(kernels) == "fine_cost_runs"
+    del kernels["fine_cost_census"]
+    assert bench.dominant_kernel(kernels) == "fine_cost_wide"
