@@ -133,10 +133,11 @@ lfsgm_status lfsgm_get_tuning(lfsgm_handle h, int32_t *row_kw, int32_t *list_cta
  * scanlines (along image borders, where the initial pass leaves whole-range windows) otherwise
  * outlast all others; the CTA's other warps wait while its first runs the narrow steps, so the
  * split pays only where a few scanlines are much longer than the rest.  The kernel that clears agg
- * lists them; when more than 256 qualify (most windows wide), none is split.  The aggregate is the
- * same bit for bit with any value.  lfsgm_get_sgm_split reads back what the caller or lfsgm_autotune
- * has set (0 also while nothing is set), lfsgm_sgm_split_used the threshold that the calls run with
- * (0: none).  Errors: LFSGM_ERR_INVALID_ARG for a negative value. */
+ * lists them; when more than 256 qualify (64 with the library's own threshold, where every scanline
+ * has a warp of its own), none is split.  The aggregate is the same bit for bit with any value.
+ * lfsgm_get_sgm_split reads back what the caller or lfsgm_autotune has set (0 also while nothing is
+ * set), lfsgm_sgm_split_used the threshold that the calls run with (0: none).
+ * Errors: LFSGM_ERR_INVALID_ARG for a negative value. */
 lfsgm_status lfsgm_set_sgm_split(lfsgm_handle h, int32_t min_wide);
 lfsgm_status lfsgm_get_sgm_split(lfsgm_handle h, int32_t *min_wide);
 lfsgm_status lfsgm_sgm_split_used(lfsgm_handle h, int32_t *min_wide);

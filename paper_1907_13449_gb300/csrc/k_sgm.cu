@@ -49,6 +49,7 @@ constexpr int kSgmWarps = 4;      // default warps (scanlines) per CTA; 2, 4 or 
 constexpr int kSplitRing = 4;     // cost rows of a split scanline's wide steps on their way (a power of two)
 constexpr int kPairFrom = 1024;   // scanlines from which on a warp may take two (twelve 5x5 x 251 x 283 side by side:
                                   // 2015 us with one, 1914 with two; 764 scanlines of 5x5 x 64^2: 20.6 and 21.0)
+constexpr int kPairPlaces = 2 * 28 * 152;   // scanlines in flight at once, two a warp
 constexpr int kSplitCap = 256;    // most scanlines split across a CTA's warps (more qualify: none is)
 
 // L rounded to a multiple of q (see above); B = C + P2 of the cell.  With M = 1.5 x 2^(floor(log2 B)
@@ -678,11 +679,11 @@ __device__ __forceinline__ void sgm_pair(const float *__restrict__ cost, const i
 // One warp per scanline, WPC warps per CTA; with split (not null), the first scap CTAs take one
 // listed scanline each with all their warps (sgm_scanline SPLIT), and the other warps skip the
 // listed ones.  split: [0] scanlines listed, [1 .. scap] the list (rs), then the wide windows of each
-// scanline and, last, of the image (count_wide); more than scap listed: none is split.  PAIR: where the
-// image has at most pair_wide (1 %) wide windows, a warp takes two scanlines (sgm_pair), and the CTAs past
-// them have nothing to do: 512^2 pixels without wide windows 174 -> 141 us, 4x4 x 720 x 1280 with 16
-// directions and 0.6 % of them 1163 -> 800 us, but with 2 % of them 212 -> 221 us and with 10 % 321 -> 425 us,
-// since both scanlines wait for the wide steps of either.
+// scanline and, last, of the image (count_wide); more than scap listed, or more than alone where every
+// scanline has its warp: none is split.  PAIR: where the image has at most pair_wide wide windows
+// (launch_fine_sgm), a warp takes two scanlines (sgm_pair), and the CTAs past them have nothing to do:
+// 512^2 pixels without wide windows 174 -> 141 us, 4x4 x 720 x 1280 with 16 directions and 0.6 % of them
+// 1163 -> 800 us; both scanlines wait for the wide steps of either.
 // Resident CTAs per SM that the register budget must allow: what the one-warp path reaches on its
 // own (72 registers without the record, 96 with it; 8 warps: 80 and 128), so that the split path
 // (more registers) does not lower the occupancy of every CTA.
@@ -710,7 +711,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
                                                                   unsigned char *__restrict__ codes,
                                                                   int *__restrict__ amin, size_t nnz_cap,
                                                                   const int *__restrict__ split, int scap,
-                                                                  int min_wide, int pair_wide) {
+                                                                  int min_wide, int alone, int pair_wide) {
     extern __shared__ __align__(16) float sm[];
     const int wib = threadIdx.x >> 5;
     // rows by slot with one sentinel slot on each side (slot -1 and slot n hold +inf), Gs + 8 floats,
@@ -722,7 +723,8 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     const float P1 = __ldg(pen), P2 = __ldg(pen + 1);
     const int total = st.cum[st.paths];
     const int nsplit = split ? __ldg(split) : 0;
-    const bool on = split && nsplit <= scap;
+    const bool paired = PAIR && __ldg(split + 1 + scap + total) <= pair_wide;
+    const bool on = split && nsplit <= (paired ? scap : alone);
     if ((int)blockIdx.x < scap) {
         if (!on || (int)blockIdx.x >= nsplit) return;
         float *bufA = sm + 4;                   // the split rows on 16-byte boundaries, Gs + 8 floats
@@ -733,7 +735,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     }
     const int gw = ((int)blockIdx.x - scap) * WPC + wib;
     if constexpr (PAIR) {
-        if (__ldg(split + 1 + scap + total) <= pair_wide) {
+        if (paired) {
             if (2 * gw >= total) return;
             const int q = 2 * gw + ((threadIdx.x >> 4) & 1);
             const int rs = q < total ? __ldg(order + q) : 0;
@@ -969,7 +971,7 @@ int sgm_split_ints(int H, int W, int paths) {
 cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, const int *cnt,
                             const long long *off, int H, int W, int G, const float *pen, float *agg,
                             int *status, const int *order, int paths, unsigned char *codes, int *amin,
-                            size_t nnz_cap, int warps_per_cta, int min_wide, const int *split, bool narrow) {
+                            size_t nnz_cap, int warps_per_cta, int min_wide, const int *split, int alone, bool narrow) {
     const int wpc = warps_per_cta == 2 || warps_per_cta == 8 ? warps_per_cta : kSgmWarps;
     const ScanTable st = make_scan_table(H, W, paths);
     const int Gs = (G + 31) & ~31;
@@ -980,6 +982,14 @@ cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, co
     const bool pair = split && narrow && !codes && st.cum[paths] >= kPairFrom && psmem * 28 <= (size_t)wpc * 224 * 1024;
     const size_t smem =
         pair ? psmem : row_floats(wpc, Gs, split, false) * sizeof(float) + (size_t)wpc * 64 * sizeof(int2) + rest;
+    // Wide windows up to which they do: a pair's time is that of its longest scanline, with the wide steps of
+    // both, so the line rises with the steps that a place in flight takes, in longest scanlines, and falls with
+    // the labels of a wide step.  One scanline a warp and two, us: 512^2, 8 directions, 401 labels, 0.9 %: 188, 181,
+    // 1.6 %: 197, 218; 121 labels, 2 %: 191, 171, 5.6 %: 183, 231; 512^2, 16 directions, 401 labels, 3.4 %: 381, 340,
+    // 5.6 %: 436, 450; 300^2, 8 directions, 201 labels, 0.9 %: 85, 88; 720 x 1280, 16 directions, 241 labels, 2 %: 1232,
+    // 817, 5.8 %: 1425, 1007.  (A line at 1 % whatever the shape left the last two at 1232 and 1425.)
+    const double steps = (double)paths * H * W / kPairPlaces / std::max(H, W);
+    const int pair_wide = (int)(std::min(1.0, std::max(0.5, 20.0 * (steps - 0.31)) / G) * H * W);
     const int scap = split ? kSplitCap : 0;
     const unsigned grid = (unsigned)(scap + (st.cum[paths] + wpc - 1) / wpc);
     // one instantiation per CTA size, each with its own register budget (launch bounds)
@@ -994,7 +1004,7 @@ cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, co
     while ((1 << lp) < paths) lp++;
     const int mk = (lp << 23) | (1 << 22);       // (23 - qsh) << 23 with qsh = 23 - log2(paths)
     kern<<<grid, 32 * wpc, smem, s>>>(cost, lo, cnt, off, H, W, Gs, pen, G, st, agg, status, order, mk, codes,
-                                      amin, nnz_cap, split, scap, min_wide, H * W / 100);
+                                      amin, nnz_cap, split, scap, min_wide, std::min(alone, scap), pair_wide);
     return cudaGetLastError();
 }
 

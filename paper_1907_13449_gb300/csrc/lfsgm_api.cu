@@ -778,6 +778,10 @@ lfsgm_status clear_split(lfsgm_ctx *h) {
         cudaMemsetAsync(h->split, 0, (size_t)sgm_split_ints(h->cfg.H, h->cfg.W, h->cfg.paths) * 4, h->stream);
     return e == cudaSuccess ? LFSGM_OK : cuda_fail(h, e, "memset");
 }
+// Most scanlines split where every scanline has its warp; with the library's own threshold 64, since the tail that
+// splitting shortens is then few scanlines: 512^2, 401 labels, 8 directions, 208 listed: 230 us unsplit, 283 split; 200
+// listed: 181 and 215 (16 directions: 316 and 334); the benchmark scenes list up to 22.
+int split_most(const lfsgm_ctx *h) { return h->sgm_split > 0 ? 256 : 64; }
 int *split_table(lfsgm_ctx *h) { return split_from(h) > 0 ? h->split : nullptr; }
 
 // Explicit penalties: zero the aggregate and list the scanlines to split.
@@ -825,7 +829,7 @@ lfsgm_status lfsgm_sgm_aggregate(lfsgm_handle h, const float *cost, const int32_
     }
     LFSGM_TRY(run(h, "fine_sgm", [&] {
         return launch_fine_sgm(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, h->fpen, agg, h->status, h->d_order,
-                               c.paths, nullptr, nullptr, 0, h->sgm_warps, split_from(h), split_table(h),
+                               c.paths, nullptr, nullptr, 0, h->sgm_warps, split_from(h), split_table(h), split_most(h),
                                2 * std::max(c.fine_radius, c.fine_radius_far) < 32);
     }));
     return LFSGM_OK;
@@ -883,7 +887,7 @@ static lfsgm_status aggregate_recording(lfsgm_handle h, const float *cost, const
     return run(h, "fine_sgm_record", [&] {
         return launch_fine_sgm(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, h->fpen, agg, h->status, h->d_order,
                                c.paths, h->b_codes, h->b_amin, (size_t)cap, h->sgm_warps,
-                               split_from(h), split_table(h));
+                               split_from(h), split_table(h), split_most(h));
     });
 }
 

@@ -151,3 +151,38 @@ def test_new_handle_gives_the_bits_of_no_split(gpu_lib, H, W, rows, cols, penalt
     gpu_lib.lfsgm_sync(h)
     gpu_lib.lfsgm_destroy(h)
     assert all(torch.equal(out[0], a) for a in out[1:])
+
+
+# a share of wide windows at which scanlines run two to a warp in images of any shape (0.3 %), and more: both forms
+@pytest.mark.parametrize("H,W,paths", [(20, 260, 16), (37, 257, 8), (330, 361, 8), (300, 310, 16)])
+@pytest.mark.parametrize("share", [0.003, 0.02, 0.3])
+def test_wide_windows_by_share_match_the_oracle(gpu_lib, H, W, paths, share):
+    G = 97
+    p, _, lo, cnt, _ = _case(H, W, paths, "narrow", G)
+    rng = np.random.default_rng(int(share * 1000) + W)
+    wide = rng.random(H * W) < share
+    cnt[wide] = rng.integers(33, 90, int(wide.sum()))
+    lo = np.minimum(lo, G - cnt).astype(np.int32)
+    off_o = oracle.offsets(cnt)
+    cost = np.random.default_rng(3).uniform(0, 30, int(off_o[-1])).astype(np.float32)
+    P1, P2 = np.float32(1.7), np.float32(9.5)
+    Cs = oracle.sgm_bounded(H, W, lo, cnt, off_o, cost.astype(np.float64), float(P1), float(P2), paths)
+    for split in (None, 0):
+        off, agg = _gpu_sgm(gpu_lib, p, cost, lo, cnt, P1, P2) if split == 0 else _new_handle_sgm(gpu_lib, p, cost, lo, cnt, P1, P2)
+        err = csr_rel_err(gather(agg, off, cnt), Cs, cnt)
+        assert err < RTOL, (split, err)
+
+
+def _new_handle_sgm(gpu_lib, p, cost, lo, cnt, P1, P2):
+    """As _gpu_sgm, on a handle whose split is not set."""
+    import torch
+    off = pad4_offsets(cnt)
+    full = np.zeros(int(off[-1]), np.float32)
+    full[np.repeat(off[:-1], cnt) + (np.arange(int(cnt.sum())) - np.repeat(np.cumsum(cnt) - cnt, cnt))] = cost
+    cd = _dev(full)
+    h = gpu_lib.lfsgm_create(p)
+    agg = torch.full_like(cd, float("nan"))
+    gpu_lib.lfsgm_sgm_aggregate(h, cd, _dev(lo, torch.int32), _dev(cnt, torch.int32), _dev(off), P1, P2, agg)
+    gpu_lib.lfsgm_sync(h)
+    gpu_lib.lfsgm_destroy(h)
+    return off, _np(agg)
