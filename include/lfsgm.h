@@ -134,7 +134,7 @@ lfsgm_status lfsgm_get_tuning(lfsgm_handle h, int32_t *row_kw, int32_t *list_cta
  * outlast all others; the CTA's other warps wait while its first runs the narrow steps, so the
  * split pays only where a few scanlines are much longer than the rest.  The kernel that clears agg
  * lists them; when more than 256 qualify (64 with the library's own threshold, where every scanline
- * has a warp of its own), none is split.  The aggregate is the same bit for bit with any value.
+ * has a warp of its own and none is much longer than the rest), none is split.  The aggregate is the same bit for bit with any value.
  * lfsgm_get_sgm_split reads back what the caller or lfsgm_autotune has set (0 also while nothing is
  * set), lfsgm_sgm_split_used the threshold that the calls run with (0: none).
  * Errors: LFSGM_ERR_INVALID_ARG for a negative value. */

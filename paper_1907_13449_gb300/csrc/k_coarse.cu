@@ -259,7 +259,8 @@ __device__ __forceinline__ void red_words(uint16_t *dst, const uint32_t *v) {
 // below 2^14; labels below 0 read 0x7fff.  The absent labels' sums overflow their halfwords,
 // but a carry only runs into higher, also absent, labels or out of the reduced word, and the
 // WTA reads labels below Lc only.
-// What bounds it: the ALU pipe (byte permutes and halfword minima run at half rate).  The step's
+// What bounds it: shared-memory, shuffle and reduction instructions (9x9 x 512^2, 100 labels, 404 us: L1 / MIO pipe
+// 82 %, mio_throttle the longest stall, issue active 74 %, ALU pipe 64 %; without the reductions about 300 us).  The step's
 // minimum is taken with both halves of the word equal (the lane's minimum and its swap), so the
 // warp's 32-bit minimum is the packed pair (m, m) and needs no unpacking; where the labels leave a
 // lane of the group empty (EDGE false), the neighbours of the first and last label come from that

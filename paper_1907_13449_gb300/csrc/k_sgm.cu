@@ -679,8 +679,9 @@ __device__ __forceinline__ void sgm_pair(const float *__restrict__ cost, const i
 // One warp per scanline, WPC warps per CTA; with split (not null), the first scap CTAs take one
 // listed scanline each with all their warps (sgm_scanline SPLIT), and the other warps skip the
 // listed ones.  split: [0] scanlines listed, [1 .. scap] the list (rs), then the wide windows of each
-// scanline and, last, of the image (count_wide); more than scap listed, or more than alone where every
-// scanline has its warp: none is split.  PAIR: where the image has at most pair_wide wide windows
+// scanline and of the image, then 1 if a scanline crosses four times as many as listed ones must
+// (count_wide); more than scap listed, or, where every scanline has its warp and none is that much longer
+// than the rest, more than alone: none is split.  PAIR: where the image has at most pair_wide wide windows
 // (launch_fine_sgm), a warp takes two scanlines (sgm_pair), and the CTAs past them have nothing to do:
 // 512^2 pixels without wide windows 174 -> 141 us, 4x4 x 720 x 1280 with 16 directions and 0.6 % of them
 // 1163 -> 800 us; both scanlines wait for the wide steps of either.
@@ -724,7 +725,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     const int total = st.cum[st.paths];
     const int nsplit = split ? __ldg(split) : 0;
     const bool paired = PAIR && __ldg(split + 1 + scap + total) <= pair_wide;
-    const bool on = split && nsplit <= (paired ? scap : alone);
+    const bool on = split && (nsplit <= (paired ? scap : alone) || (nsplit <= scap && __ldg(split + 2 + scap + total) != 0));
     if ((int)blockIdx.x < scap) {
         if (!on || (int)blockIdx.x >= nsplit) return;
         float *bufA = sm + 4;                   // the split rows on 16-byte boundaries, Gs + 8 floats
@@ -775,7 +776,9 @@ __device__ __forceinline__ void count_wide(unsigned wide, int p0, int W, int H, 
         dir_of(r, dx, dy);
         const int base = scan_base(st, r);
         const int q = scan_index_d(dx, dy, x, y, H, W);
-        if (atomicAdd(tab + 1 + kSplitCap + base + q, 1) == min_wide - 1) {
+        const int before = atomicAdd(tab + 1 + kSplitCap + base + q, 1);
+        if (before == 4 * min_wide - 1) tab[2 + kSplitCap + st.cum[st.paths]] = 1;
+        if (before == min_wide - 1) {
             const int pos = atomicAdd(tab, 1);
             if (pos < kSplitCap) tab[1 + pos] = (q << 4) | r;
         }
@@ -965,7 +968,7 @@ void build_scan_order(int H, int W, int paths, std::vector<int> &order) {
 }
 
 int sgm_split_ints(int H, int W, int paths) {
-    return 1 + kSplitCap + make_scan_table(H, W, paths).cum[paths] + 1;
+    return 1 + kSplitCap + make_scan_table(H, W, paths).cum[paths] + 2;
 }
 
 cudaError_t launch_fine_sgm(cudaStream_t s, const float *cost, const int *lo, const int *cnt,

@@ -778,9 +778,10 @@ lfsgm_status clear_split(lfsgm_ctx *h) {
         cudaMemsetAsync(h->split, 0, (size_t)sgm_split_ints(h->cfg.H, h->cfg.W, h->cfg.paths) * 4, h->stream);
     return e == cudaSuccess ? LFSGM_OK : cuda_fail(h, e, "memset");
 }
-// Most scanlines split where every scanline has its warp; with the library's own threshold 64, since the tail that
-// splitting shortens is then few scanlines: 512^2, 401 labels, 8 directions, 208 listed: 230 us unsplit, 283 split; 200
-// listed: 181 and 215 (16 directions: 316 and 334); the benchmark scenes list up to 22.
+// Most scanlines split where every scanline has its warp; with the library's own threshold 64, unless some are four
+// times as long as listed ones must be: splitting shortens the tail of a few.  512^2, 401 labels, 8 directions, 208
+// listed: 230 us unsplit, 283 split; 200 listed: 181 and 215 (16 directions: 316 and 334); with two scanlines of 147 among
+// them (recording): 406 unsplit, 320 split.
 int split_most(const lfsgm_ctx *h) { return h->sgm_split > 0 ? 256 : 64; }
 int *split_table(lfsgm_ctx *h) { return split_from(h) > 0 ? h->split : nullptr; }
 
