@@ -40,7 +40,11 @@ PENALTY_NOTE = "P1 = 0.05 mean cost, P2 = 0.5 mean cost (coarse: per arm, intege
 
 # DRAM bytes (read + write) per launch from one ncu capture of the bench workload, with the
 # SHA-256 prefix of the kernel's source at capture time; a changed source reports null.
-NCU_TRAFFIC = {}   # no capture of the bench workload with the present row kernel (k_fine_rows.cu)
+NCU_TRAFFIC = {
+    "fine_cost": {"bytes": 335231232, "workload": "bench", "channels": 1,
+                  "source": "paper_1907_13449_gb300/csrc/k_fine_rows.cu",
+                  "sha256_16": "1fa045412c4de22f"},
+}
 
 
 # The kernels of the cost and SGM stages (derived penalties), by their names in lfsgm_kernel_times.

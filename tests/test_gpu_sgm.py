@@ -186,3 +186,36 @@ def _new_handle_sgm(gpu_lib, p, cost, lo, cnt, P1, P2):
     gpu_lib.lfsgm_sync(h)
     gpu_lib.lfsgm_destroy(h)
     return off, _np(agg)
+
+
+# 160 scanlines that cross 26 wide windows each: too many to split on a new handle, unless one crosses 96 (the whole row)
+@pytest.mark.parametrize("long_row", [False, True])
+@pytest.mark.parametrize("record", [False, True])
+def test_many_listed_scanlines_give_the_bits_of_no_split(gpu_lib, long_row, record):
+    import torch
+    H, W, G = 300, 260, 75
+    rng = np.random.default_rng(9)
+    lo = rng.integers(0, G, (H, W)).astype(np.int32)
+    cnt = np.minimum(rng.integers(1, 33, (H, W)), G - lo).astype(np.int32)
+    for y in range(80):
+        x = 3 * y % 230
+        lo[y, x:x + 26], cnt[y, x:x + 26] = 0, G
+    if long_row:
+        lo[200], cnt[200] = 0, G
+    lo, cnt = lo.ravel(), cnt.ravel()
+    off = pad4_offsets(cnt)
+    cost = rng.uniform(0, 30, int(off[-1])).astype(np.float32)
+    p = lfsynth.LFParams(U=3, V=3, H=H, W=W, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=40, fine_labels=G,
+                         fine_radius=5)
+    d = [_dev(cost), _dev(lo, torch.int32), _dev(cnt, torch.int32), _dev(off)]
+    h = gpu_lib.lfsgm_create(p)
+    out = []
+    for min_wide in (None, 0, 24):
+        if min_wide is not None:
+            gpu_lib.lfsgm_set_sgm_split(h, min_wide)
+        agg = torch.full_like(d[0], float("nan"))
+        (gpu_lib.lfsgm_sgm_aggregate_record if record else gpu_lib.lfsgm_sgm_aggregate)(h, *d, 1.5, 9.0, agg)
+        out.append(agg)
+    gpu_lib.lfsgm_sync(h)
+    gpu_lib.lfsgm_destroy(h)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
