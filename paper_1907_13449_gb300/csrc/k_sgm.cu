@@ -152,9 +152,9 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                                              int wib, float *cring = nullptr, int cstride = 0) {
     const int lane = threadIdx.x & 31;
     const int r = rs & 15, s = rs >> 4;
-    const int dx = dir_dx(r), dy = dir_dy(r);
-    int x0, y0;
-    scan_start(r, s, H, W, x0, y0);
+    int dx, dy, x0, y0;
+    dir_of(r, dx, dy);
+    scan_start_d(dx, dy, s, H, W, x0, y0);
     const int len = scan_steps(x0, y0, dx, dy, H, W);
     unsigned char *code = REC ? codes + (size_t)r * nnz_cap : nullptr;
     int *am = REC ? amin + (size_t)r * H * W : nullptr;
@@ -396,7 +396,7 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                 // one warp: four vectors of four labels a lane per round, their cost loads in flight together
                 // (512^2 pixels, windows of 401 labels at 10 % and 30 % of them: 282 and 503 us, with a label a lane
                 // 303 and 565)
-                if constexpr (!SPLIT) {
+                if constexpr (!SPLIT && !REC) {
                     const bool same = l == plo && n == pn;
                     const unsigned top = (unsigned)pn + 1u;
                     for (int jr = 4 * lane; jr < n; jr += 512) {
@@ -411,6 +411,66 @@ __device__ __forceinline__ void sgm_scanline(const float *__restrict__ cost, con
                             wide_cells<REC>(c4[u], jr + 128 * u, n, l, plo, pn, same, top, bufA, m, P1, P2, mk, agg + o,
                                             REC ? code + o : nullptr, lmin, lslot, bufB);
                         }
+                    }
+                }
+                // sixteen of this warp's 32-label chunks per round: their cost loads are in flight
+                // together, and every chunk reads the predecessor row before any chunk stores its own
+                // (the compiler cannot tell bufA from bufB, so a store between them would order the
+                // chunks one after another)
+                constexpr int CS = 32;                 // slot stride between the chunks
+                if constexpr (REC && !SPLIT)
+                for (int j0 = lane; j0 < n; j0 += 16 * CS) {
+                    float cc[16];
+#pragma unroll
+                    for (int u = 0; u < 16; u++) cc[u] = j0 + CS * u < n ? __ldg(cost + o + j0 + CS * u) : 0.f;
+                    if (pn != 0) {
+                        // predecessor slot s read at row[s + 1] with s + 1 clamped (unsigned) to
+                        // pn + 1: any slot outside [0, pn) lands on a sentinel (+inf), so an absent
+                        // label drops out of the minimum (labels j >= n read in-bounds slots too)
+                        const unsigned top = (unsigned)pn + 1u;
+                        const float *row = bufA - 1;
+                        auto step = [&](int u, float v0, float vm, float vp) {
+                            const float t = fminf(fminf(m + P2, v0), fminf(vm, vp) + P1);
+                            code[o + j0 + CS * u] = t == m + P2 ? 3 : (t == v0 ? 0 : (t == vm + P1 ? 1 : 2));
+                            const float Ln = cc[u] + (t - m);
+                            // the cell's cost cc[u] bounds its path costs (the global atomic does
+                            // not order the shared-memory reads of the other chunks)
+                            atomicAdd(agg + o + j0 + CS * u, det_addend(Ln, cc[u] + P2, mk));
+                            cc[u] = Ln;
+                        };
+                        if (l == plo && n == pn) {
+                            // the same window as the predecessor (a run of whole-range windows):
+                            // slot j's neighbours are slots j - 1 and j + 1, and the sentinels at
+                            // slots -1 and pn stand in for the absent ones
+                            const float *q = bufA + j0;
+#pragma unroll
+                            for (int u = 0; u < 16; u++) {
+                                if (j0 + CS * u >= n) break;
+                                step(u, q[CS * u], q[CS * u - 1], q[CS * u + 1]);
+                            }
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 16; u++) {
+                                if (j0 + CS * u >= n) break;
+                                const unsigned k1 = (unsigned)(l + j0 + CS * u - plo + 1);
+                                step(u, row[min(k1, top)], row[min(k1 - 1u, top)], row[min(k1 + 1u, top)]);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 16; u++) {
+                            if (j0 + CS * u >= n) break;
+                            atomicAdd(agg + o + j0 + CS * u, det_addend(cc[u], cc[u] + P2, mk));
+                            code[o + j0 + CS * u] = 4;
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 16; u++) {
+                        const int j = j0 + CS * u;
+                        if (j >= n) break;
+                        bufB[j] = cc[u];
+                        if (cc[u] < lmin) lslot = j;      // a lane's slots ascend: its first minimum
+                        lmin = fminf(lmin, cc[u]);
                     }
                 }
                 if (SPLIT) {
@@ -722,7 +782,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     int2 *ring = reinterpret_cast<int2 *>(sm + rows), *meta = ring + wib * 64;
     float *xm = sm + rows + (PAIR ? 2 : 1) * WPC * 128;
     const float P1 = __ldg(pen), P2 = __ldg(pen + 1);
-    const int total = st.cum[st.paths];
+    const int total = st.paths == 8 ? st.cum[8] : st.cum[16];   // (no run-time index, see scan_base)
     const int nsplit = split ? __ldg(split) : 0;
     const bool paired = PAIR && __ldg(split + 1 + scap + total) <= pair_wide;
     const bool on = split && (nsplit <= (paired ? scap : alone) || (nsplit <= scap && __ldg(split + 2 + scap + total) != 0));
@@ -748,7 +808,7 @@ __global__ void __launch_bounds__(32 * WPC, sgm_min_ctas(REC, WPC)) fine_sgm_ker
     }
     if (gw >= total) return;
     const int rs = __ldg(order + gw);            // longest scanlines first
-    if (on && __ldg(split + 1 + scap + st.cum[rs & 15] + (rs >> 4)) >= min_wide) return;
+    if (on && __ldg(split + 1 + scap + scan_base(st, rs & 15) + (rs >> 4)) >= min_wide) return;
     float *bufA = sm + (size_t)wib * 2 * (Gs + 8) + 4;
     sgm_scanline<REC, false, 1>(cost, lo, cnt, off, H, W, P1, P2, G, agg, status, rs, mk, codes, amin, nnz_cap,
                                 bufA, bufA + (Gs + 8), meta, xm, wib);
