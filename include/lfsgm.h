@@ -129,7 +129,8 @@ lfsgm_status lfsgm_get_tuning(lfsgm_handle h, int32_t *row_kw, int32_t *list_cta
  * windows wider than 32 labels runs on all the warps of one CTA, which share each wide step's
  * labels, four to a thread, instead of on one warp (0: none does, and every scanline has a warp of
  * its own).  While it is not set, the library takes 24 for images of at least 256 pixels in a
- * direction, and none for smaller ones and for searches over the whole range.  Such
+ * direction, and none for smaller ones, for searches over the whole range and where the regular
+ * windows (fine_radius) are wider than 32 labels.  Such
  * scanlines (along image borders, where the initial pass leaves whole-range windows) otherwise
  * outlast all others; the CTA's other warps wait while its first runs the narrow steps, so the
  * split pays only where a few scanlines are much longer than the rest.  The kernel that clears agg

@@ -254,16 +254,19 @@ lfsgm_status ensure_workspace(lfsgm_ctx *h) {
 bool census_only(const lfsgm_ctx *h) { return h->cfg.w_l2 == 0.f && h->C == 1; }
 int *large_flag(lfsgm_ctx *h) { return census_only(h) ? h->wide_count + 2 : nullptr; }
 
+// Windows of at most 32 labels where the initial map holds.
+bool narrow_windows(const lfsgm_ctx *h) { return 2 * std::max(h->cfg.fine_radius, h->cfg.fine_radius_far) < 32; }
+
 // Windows wider than 32 labels from which on a scanline runs split across a CTA (0: none does).  Where
 // the caller has set no threshold: 24, unless scanlines are short (a scanline of 256 steps with 24 such
-// windows takes about as long as one of 340 without) or every window is the whole range (then all are
-// alike).  Two scanlines of 9x9 x 512^2 cross 147 windows of 401 labels each and outlast all others:
+// windows takes about as long as one of 340 without) or the regular windows are wide or the whole range
+// (then all are alike, and counting them takes 35 us of 5x5 x 300 x 400).  Two scanlines of 9x9 x 512^2 cross 147 windows of 401 labels each and outlast all others:
 // 297 us without, 242 with the split (24, 48 and 96 alike, 215 with vectors of four labels; recording 382
 // and 313); the same time without such scanlines.  8 or 12 list more than the table holds.
 int split_from(const lfsgm_ctx *h) {
     const lfsgm_config &c = h->cfg;
     if (h->sgm_split >= 0) return h->sgm_split;
-    return !c.boundless && std::max(c.H, c.W) >= 256 ? 24 : 0;
+    return !c.boundless && narrow_windows(h) && std::max(c.H, c.W) >= 256 ? 24 : 0;
 }
 
 int max_arm_views(const lfsgm_ctx *h) {
@@ -831,7 +834,7 @@ lfsgm_status lfsgm_sgm_aggregate(lfsgm_handle h, const float *cost, const int32_
     LFSGM_TRY(run(h, "fine_sgm", [&] {
         return launch_fine_sgm(s, cost, lo, cnt, o, c.H, c.W, c.fine_labels, h->fpen, agg, h->status, h->d_order,
                                c.paths, nullptr, nullptr, 0, h->sgm_warps, split_from(h), split_table(h), split_most(h),
-                               2 * std::max(c.fine_radius, c.fine_radius_far) < 32);
+                               narrow_windows(h));
     }));
     return LFSGM_OK;
 }

@@ -219,3 +219,12 @@ def test_many_listed_scanlines_give_the_bits_of_no_split(gpu_lib, long_row, reco
     gpu_lib.lfsgm_sync(h)
     gpu_lib.lfsgm_destroy(h)
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("radius,far,own", [(15, 0, 24), (16, 0, 0), (5, 16, 0)])
+def test_no_split_of_its_own_where_the_regular_windows_are_wide(gpu_lib, radius, far, own):
+    p = lfsynth.LFParams(U=3, V=3, H=20, W=260, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=40, fine_labels=75,
+                         fine_radius=radius, fine_radius_far=far)
+    h = gpu_lib.lfsgm_create(p)
+    assert gpu_lib.lfsgm_sgm_split_used(h) == own
+    gpu_lib.lfsgm_destroy(h)
