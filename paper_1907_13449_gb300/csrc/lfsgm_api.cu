@@ -744,7 +744,7 @@ lfsgm_status cost_volume_impl(lfsgm_handle h, const float *views, const int32_t 
                                    h->N, h->status);
         }));
     }
-    if (census_only(h) && h->rows_maps)
+    if (census_only(h) && h->rows_maps && c.fine_labels > 32)      // (a marked run's windows are wider than 32 labels)
         LFSGM_TRY(run(h, "fine_cost_runs", [&] {
             return launch_census_runs(s, h->cen_pad, h->rows.P, h->rows.Wp, h->rows.Hp, h->d_ctab, c.fine_labels,
                                       h->nviews, c.H, c.W, h->ref, h->marks, (const long long *)off, c.w_census, cost);

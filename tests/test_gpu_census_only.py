@@ -60,3 +60,24 @@ def test_non_finite_views_keep_the_full_form(gpu_lib):
     got = _cost(gpu_lib, p, views, lo, cnt, off)
     bad = np.isnan(got)
     assert bad.any() and not bad.all()
+
+
+def test_no_launch_for_runs_that_cannot_be(gpu_lib):
+    """Up to 32 fine labels no window is wider than 32, so no run is marked: its kernel is left out; the costs are
+    those of the oracle."""
+    import torch
+    p = lfsynth.LFParams(U=4, V=3, H=21, W=70, census_w=5, dmin=-2.0, dmax=2.0, coarse_labels=40, fine_labels=32,
+                         fine_radius=3, w_l2=0.0, w_census=1.0, boundless=1)
+    views = lfsynth.random_views(4, 3, p.H, p.W, seed=8)
+    L = gpu_lib.LightFieldDepth(p)
+    vd = torch.from_numpy(views).cuda()
+    L.initial(vd)
+    gpu_lib.lfsgm_set_profiling(L.h, True)
+    L.cost_volume(vd)
+    gpu_lib.lfsgm_sync(L.h)
+    assert "fine_cost_runs" not in [n for n, _ in gpu_lib.lfsgm_kernel_times(L.h)]
+    got = L.cost.cpu().numpy()[:p.N * 32].reshape(p.N, 32)
+    L.close()
+    lo, cnt = np.zeros(p.N, np.int32), np.full(p.N, 32, np.int32)
+    _, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    assert np.array_equal(got.astype(np.float64).ravel(), ref)
