@@ -521,7 +521,11 @@ cudaError_t launch_coarse_sgm(cudaStream_t s, const void *cost, bool cost8, int 
     const long long warps = ((long long)st.cum[paths] * narms + sub - 1) / sub;
     const int block = 128;
     const unsigned grid = (unsigned)((warps * 32 + block - 1) / block);
-#define LFSGM_SGM(LPT, B, SUB, E) coarse_sgm_kernel<LPT, B, SUB, E><<<grid, block, 0, s>>>(cost, H, W, Lc, Lcd, pen, st.cum[paths], narms, sum, order)
+    // Above 128 labels six CTAs per SM (38 KB each with their rings): the costs and sums of the scanlines in flight
+    // outgrow L2.  512^2, 4 arms, 192 and 256 labels: 1140 and 1571 us with the ten that the registers allow, 981 and 1414
+    // with six, 980 and 1416 with five, 1010 and 1450 with four; 200^2: 189, 186, 187, 182.
+    const size_t room = lpt == 8 ? 38 * 1024 - (size_t)4 * 8 * 32 * (cost8 ? 8 : 16) : 0;
+#define LFSGM_SGM(LPT, B, SUB, E) coarse_sgm_kernel<LPT, B, SUB, E><<<grid, block, room, s>>>(cost, H, W, Lc, Lcd, pen, st.cum[paths], narms, sum, order)
 #define LFSGM_SGM4(LPT, SUB)                                                                    \
     do {                                                                                        \
         if (cost8) { if (edge) LFSGM_SGM(LPT, true, SUB, true); else LFSGM_SGM(LPT, true, SUB, false); } \
