@@ -104,11 +104,12 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity) {
 // One CTA per block of 32 x 8 pixels, a warp per row: every row's range (the start, of its windows'
 // starts, whose kw labels hold the most of them; ties: the lowest), then the tasks of the block.  Task
 // b (b < nblk) is block b's first (no pixels: none); further ones take the slots from nblk on (*extra
-// of them; at most eight tasks a block).  Rows are grouped greedily: the start G0 whose kwt labels hold the most pending rows.  Wide windows and those outside
-// their row's range go to the list, in 32-label chunks.
+// of them; at most eight tasks a block).  Rows are grouped greedily: the start G0 whose kwt labels hold the
+// most pending rows, `most` of them at most.  Wide windows and those outside their row's range go to the list, in
+// 32-label chunks.
 __global__ void __launch_bounds__(32 * kBlkH) row_tasks_kernel(const int *__restrict__ lo, const int *__restrict__ cnt,
                                                                const long long *__restrict__ off, int G, int H, int W,
-                                                               int kw, int kwt, int nblk, RowTask *__restrict__ tasks,
+                                                               int kw, int kwt, int most, int nblk, RowTask *__restrict__ tasks,
                                                                int *__restrict__ extra, int2 *__restrict__ list,
                                                                int *__restrict__ list_count, int *__restrict__ status,
                                                                const int *__restrict__ large,
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(32 * kBlkH) row_tasks_kernel(const int *__rest
             const int src = __ffs(__ballot_sync(0xffffffffu, cand && key == top)) - 1;
             const int G0 = __shfl_sync(0xffffffffu, qg, src);
             set = __shfl_sync(0xffffffffu, set, src);
+            while (__popc(set) > most) set &= ~(1u << (31 - __clz(set)));
             int slot = b;
             if (k > 0) {
                 slot = nblk;
@@ -707,13 +709,23 @@ bool encode_fine_rows_maps(RowPlanHost *ph, const float *views_pad, const uint64
     return true;
 }
 
+// Small images: fewer rows a task, so that the tasks are spread over the 152 SMs (up to two on each), instead of eight
+// busy warps on few of them.  us, eight rows / up to 152 tasks / 304 / 456: 9x9 x 51 x 87 (21 blocks) 253, 219, 228, 228 (a
+// warp per row with its own tile: 227); 9x9 x 160 x 192 (120 blocks) 156, 158, 140, 140; 9x9 x 64^2 in colour 313, 270, 270, 270;
+// 15x15 x 104 x 89 (39 blocks) 919, 826, 846, 1555 (704); 15x15 x 128^2 (64 blocks) 322, 342, 348, 350 (407).
+static int rows_a_task(int nblk) {
+    int rows = kBlkH;
+    while (rows > 1 && kBlkH / rows * nblk * 2 <= 304) rows /= 2;
+    return rows;
+}
+
 cudaError_t launch_row_tasks(cudaStream_t s, const RowPlanHost *ph, int G, int H, int W, const int *lo, const int *cnt,
                              const long long *off, RowTask *tasks, int *extra, int *status, int2 *list,
                              int *list_count, const int *large, unsigned char *marks) {
     RowPlan pl;
     memcpy(&pl, ph->raw, sizeof(pl));
     const int nblk = row_blocks(H, W);
-    row_tasks_kernel<<<nblk, 32 * kBlkH, 0, s>>>(lo, cnt, off, G, H, W, pl.kw, pl.kwt, nblk, tasks, extra, list, list_count,
+    row_tasks_kernel<<<nblk, 32 * kBlkH, 0, s>>>(lo, cnt, off, G, H, W, pl.kw, pl.kwt, rows_a_task(nblk), nblk, tasks, extra, list, list_count,
                                                     status, large, marks);
     return cudaGetLastError();
 }

@@ -177,3 +177,31 @@ def test_ranges_whose_boxes_just_fit_take_the_row_kernel(gpu_lib):
     L.close()
     off_o, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
     assert csr_rel_err(gather(got, off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
+
+
+# images of more than 152 blocks, whose tasks are of up to eight rows (fewer in smaller ones), with ragged edges
+@pytest.mark.parametrize("channels", [1, 3])
+@pytest.mark.parametrize("kind", ["even", "mixed"])
+def test_tasks_of_eight_rows_match_the_oracle(gpu_lib, kind, channels):
+    import torch
+    H, W, G = 203, 205, 121
+    p = lfsynth.LFParams(U=3, V=4, H=H, W=W, census_w=5, dmin=-3.0, dmax=3.0, coarse_labels=16, fine_labels=G,
+                         fine_radius=7, channels=channels)
+    rng = np.random.default_rng(20 + channels)
+    views = lfsynth.random_views(p.U, p.V, H, W, seed=21, channels=channels)
+    y, x = np.mgrid[0:H, 0:W]
+    lo = (40 + (x + y) % 3).ravel() if kind == "even" else rng.integers(0, G, H * W)
+    cnt = np.full(H * W, 31) if kind == "even" else np.where(rng.random(H * W) < 0.1, G, rng.integers(1, 33, H * W))
+    lo = lo.astype(np.int32)
+    cnt = np.minimum(cnt, G - lo).astype(np.int32)
+    off = pad4_offsets(cnt)
+    L = gpu_lib.LightFieldDepth(p)
+    L.lo.copy_(torch.from_numpy(lo))
+    L.cnt.copy_(torch.from_numpy(cnt))
+    L.off.copy_(torch.from_numpy(off))
+    L.cost_volume(torch.from_numpy(views).cuda())
+    gpu_lib.lfsgm_sync(L.h)
+    got = L.cost.cpu().numpy()
+    L.close()
+    off_o, ref = oracle.cost_volume(oracle.make_cfg(p), views, lo, cnt)
+    assert csr_rel_err(gather(got, off, cnt), gather(ref, off_o, cnt), cnt) <= RTOL
